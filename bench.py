@@ -125,7 +125,7 @@ def fp64_alu_roofline(workload: str, facet_ms: float, facets: int | None = None,
     depends on the loading state (which branch of the law each facet takes: 503 flops per facet on
     the tension cube, 297.5 on the confined-compression headline), so a workload without its own
     capture reports null rather than another workload's count scaled."""
-    fl = recorded_traffic("facet_kernel", workload, "fp64", "fp64_flops_per_launch")
+    fl = recorded_traffic("facet_edge_kernel", workload, "fp64", "fp64_flops_per_launch")
     if fl is None or not facet_ms:
         return None
     peak = fp64_peak_tflops(sm_count, sm_mhz)
@@ -391,7 +391,7 @@ def run_leg(name, wl, spec, bc, prec, steps, warmup, preroll, stream, flush_buf,
     ms_step = tot / steps
     fb, gb = facet_pass_bytes(F, T, N, r), gather_pass_bytes(T, N, r)
     ref = STORED_LAYOUT_BYTES_PER_FACET[prec]
-    kern = "facet_warp_kernel" if prec == "mixed" else "facet_kernel"
+    kern = "facet_warp_kernel" if prec == "mixed" else "facet_edge_kernel"
     return {
         "workload": name, "precision": prec, "steps": steps, "value": job_value(world, F, steps, tot),
         "ms_per_step": ms_step, "dt_s": wl.dt,

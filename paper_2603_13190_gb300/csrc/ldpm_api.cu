@@ -243,7 +243,7 @@ void free_model(ldpm_ctx *h)
                     h->dm.geo,
                     h->dm.hist, h->dm.fout, h->dm.tvc, h->dm.ent, h->dm.row, h->dm.stab, h->dm.tile_spec, h->dm.law, h->dm.spec,
                     h->dm.step, h->dm.flag, h->d_partial, h->d_out16, h->dm.pf, h->d_umap, h->d_scratch, h->d_ticket,
-                    h->d_pmap, h->pctl.arrive, h->pctl.status};
+                    h->d_pmap, h->pctl.arrive, h->pctl.status, h->dm.frame, h->dm.grad};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->h_out16) cudaFreeHost(h->h_out16);
@@ -1032,6 +1032,10 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
         rc = upload_facets<double>(raw, H, Fint);
     if (rc) return rc;
     if ((rc = update_law(raw))) return rc;
+    if (h->prec == LDPM_FP64) {
+        if ((rc = dalloc(&dm.frame, 96 * (size_t)T)) || (rc = dalloc(&dm.grad, 9 * (size_t)T))) return rc;
+        CU(launch_frames(dm, h->stream));
+    }
     // ---- time step: given, or dt_factor * 2 / sqrt(lambda_max)
     bool need = false;
     for (int s = 0; s < n; ++s) need |= !(opts[s].dt > 0);
@@ -2058,6 +2062,7 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
         for (int k3 = 0; k3 < 3; ++k3)
             if (src[k3])
                 for (int32_t k = 0; k < S.F; ++k) v[4 * (size_t)S.fmap[k] + k3] = src[k3][k];
+        for (int64_t f = 0; f < Fint; ++f) v[4 * f + 3] = 1.0 / v[4 * f + 1];
         if (!h->dm.pf) {
             int rc = h->prec == LDPM_MIXED ? dalloc((float4 **)&h->dm.pf, (size_t)Fint)
                                            : dalloc((double4a **)&h->dm.pf, (size_t)Fint);

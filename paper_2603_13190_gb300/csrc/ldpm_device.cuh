@@ -36,6 +36,12 @@ __device__ __forceinline__ V3<R> cross(V3<R> a, V3<R> b)
     return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
 
+// w + a x b
+__device__ __forceinline__ V3<double> add_cross(V3<double> w, V3<double> a, V3<double> b)
+{
+    return {fma(a.y, b.z, fma(-a.z, b.y, w.x)), fma(a.z, b.x, fma(-a.x, b.z, w.y)), fma(a.x, b.y, fma(-a.y, b.x, w.z))};
+}
+
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
 
@@ -192,6 +198,109 @@ __device__ __forceinline__ void facet_law(const LawConst<R> &c, R l, V3<R> e, V3
     tN = tn;
     tM = tm;
     tL = tl;
+}
+
+// ------------------------------------------------------------------------------------------------
+// FP64 form of the law for the edge-tile facet pass.  GB300 issues one FP64 warp instruction per ~64
+// cycles and sub-partition, comparisons included, while the FP32 and integer pipes are all but idle
+// there.  So comparisons are made on the bit patterns (order_bits), and whether a boundary of the law
+// (softening, friction) can be reached at all is decided in FP32 with a margin far above FP32's
+// rounding; only where the answer is "perhaps" is the boundary evaluated, in FP64.  The results are
+// those of facet_law up to the rounding of FP64.
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float d2f_trunc(double x);
+// Signed integer with the order of x among numbers >= 0; negative numbers (and -0) map below 0.
+__device__ __forceinline__ long long order_bits(double x) { return __double_as_longlong(x); }
+
+// Parameters of one facet: E0, alpha, 1 / alpha, sigma_t (the facet's own or the material's).
+struct FacetPar64 {
+    double E0, alpha, inv_alpha, sigma_t;
+};
+
+// Fracture boundary sigma_bt (App. A.1): strain eN > 0, aT2 = alpha e_T^2, 1 / e, e_max, and
+// ht = 2 l / (l_t - l), so that H_t = E0 ht.
+__device__ __forceinline__ double fracture_boundary64(const LawConst<double> &c, const FacetPar64 &f, double eN,
+                                                      double aT2, double inv_e, double emax, double ht)
+{
+    const double saT = sqrt(aT2);
+    const double sn = eN * inv_e, cs = saT * inv_e;
+    const double sigma0 = 2.0 * f.sigma_t / (sn + sqrt(sn * sn + f.alpha * c.four_over_r2 * cs * cs));
+    const double over = emax - sigma0 / f.E0;
+    if (order_bits(over) <= 0) return sigma0;  // not softened yet
+    const double Hs = c.r_s * f.E0 * f.inv_alpha;
+    const double H0 = Hs + (f.E0 * ht - Hs) * powpos_(atan2(eN, saT) * (2.0 / kPi), c.n_t);
+    return sigma0 * exp(-H0 * over / sigma0);
+}
+
+// A lower bound of it in FP32.  The margins: 1e-4 on sigma_0, on H_0 and on the exponent, 1e-6 of e_max
+// on <e_max - e_0> and of H_s + H_t on H_0 (differences of FP32 numbers).  NaN where FP32 cannot hold
+// the operands, which the caller takes as "perhaps".
+__device__ __forceinline__ float fracture_floor32(float E0, float four_a_r2, float Hs, float sigma_t, float n_t,
+                                                  float eN, float aT2, float inv_e, float emax, float ht)
+{
+    const float saT = sqrtf(aT2);
+    const float sn = eN * inv_e, cs = saT * inv_e;
+    const float s0 = 0.9999f * 2.0f * sigma_t / (sn + sqrtf(sn * sn + four_a_r2 * cs * cs));
+    const float over = emax - s0 / E0 + 1e-6f * emax;
+    if (over <= 0.0f) return s0;
+    const float Ht = E0 * ht;
+    const float H0 = 1.0001f * (Hs + (Ht - Hs) * powpos_(atan2f(eN, saT) * (float)(2.0 / kPi), n_t)) + 1e-6f * (Hs + Ht);
+    return 0.9999f * s0 * exp_(-1.0001f * H0 * over / s0);
+}
+
+// Compression and friction (App. A.2, A.3) of one facet, eN <= 0.  The trial: t in, the elastic trial
+// out, with t_N <= 0 applied where that is all.  Returns whether a boundary may be reached, in which
+// case compression_return64 has to follow.
+__device__ __forceinline__ bool compression_trial64(const LawConst<double> &c, const FacetPar64 &f, V3<double> de,
+                                                    V3<double> &t)
+{
+    const double ENc = order_bits(-t.x) <= order_bits(c.sigma_c0) ? f.E0 : c.Ed_E0 * f.E0;
+    const double aE = f.alpha * f.E0;
+    t = {t.x + ENc * de.x, t.y + aE * de.y, t.z + aE * de.z};
+    // H_c >= 0: sigma_bc >= sigma_c0, so a trial above -sigma_c0 is inside
+    if (!(c.Hc0_E0 >= 0.0 && c.Hc1_E0 >= 0.0 && order_bits(-t.x) <= order_bits(c.sigma_c0))) return true;
+    const float tn = fminf(d2f_trunc(t.x), 0.0f);
+    // FP32 lower bound of sigma_bs: the rounding of each of its four terms is below 1e-6 of that term
+    const float ss = d2f_trunc(c.r_st * f.sigma_t), md = d2f_trunc(c.mu_diff_sN0), mi = d2f_trunc(c.mu_inf) * tn,
+                me = md * exp_(tn * d2f_trunc(c.inv_sigma_N0));
+    const float low = (ss + md - mi - me) - 1e-5f * (ss + fabsf(md) + fabsf(mi) + fabsf(me));
+    const float tm = d2f_trunc(t.y), tl = d2f_trunc(t.z);
+    if (!(1.00001f * (tm * tm + tl * tl) <= low * low && low > 0.0f)) return true;
+    t.x = order_bits(t.x) > 0 ? 0.0 : t.x;
+    return false;
+}
+
+// The boundaries of a trial t: -sigma_bc <= t_N <= 0, then the radial return of the shear traction.
+__device__ __forceinline__ void compression_return64(const LawConst<double> &c, const FacetPar64 &f, double eN,
+                                                     double eV, V3<double> &t)
+{
+    double sigma_bc = c.sigma_c0;
+    const double ec0 = c.sigma_c0 / f.E0, eD = eN - eV;
+    const double eDV = eV + c.beta * eD;
+    if (order_bits(-eDV) > order_bits(ec0)) {  // below, <-e_DV - e_c0> = 0 and H_c does not matter
+        const double eV0 = c.kc3 * ec0, ec1 = c.kc0 * ec0, absD = fabs(eD);
+        const double rDV = order_bits(eV) <= 0 ? -absD / (eV - eV0) : absD / eV0;
+        const double mac = rDV - c.kc1 > 0.0 ? rDV - c.kc1 : 0.0;
+        const double Hc1 = c.Hc1_E0 * f.E0;
+        const double Hc = (c.Hc0_E0 * f.E0 - Hc1) / (1.0 + c.kc2 * mac) + Hc1;
+        if (-eDV <= ec1) {
+            sigma_bc = c.sigma_c0 + (-eDV - ec0) * Hc;
+        } else {
+            const double sigma_c1 = c.sigma_c0 + (ec1 - ec0) * Hc;
+            sigma_bc = sigma_c1 * exp((-eDV - ec1) * Hc / sigma_c1);
+        }
+    }
+    double tn = t.x < -sigma_bc ? -sigma_bc : t.x;
+    tn = order_bits(tn) > 0 ? 0.0 : tn;
+    const double tau2 = t.y * t.y + t.z * t.z;
+    const double sigma_bs =
+        c.r_st * f.sigma_t + c.mu_diff_sN0 - c.mu_inf * tn - c.mu_diff_sN0 * exp(tn * c.inv_sigma_N0);
+    if (tau2 > sigma_bs * sigma_bs) {
+        const double s = sigma_bs * rsqrt(tau2);
+        t.y *= s;
+        t.z *= s;
+    }
+    t.x = tn;
 }
 
 template <class R>

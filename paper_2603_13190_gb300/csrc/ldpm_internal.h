@@ -13,7 +13,11 @@
 //   tet    [T]     int4 particle ids of the 4 vertices (-1: padding tetrahedron)
 //   geo    [12T]   R4   c_a (arm from the edge's first vertex to the facet centroid), projected area A
 //   hist   [12T]   R4   t_N, t_M, t_L, e_max
-//   pf     [12T]   R4   optional per-facet E0, alpha, sigma_t, 0 (null: the material's values)
+//   pf     [12T]   R4   optional per-facet E0, alpha, sigma_t, 1/alpha (null: the material's values)
+//   frame  [6T][16] f64 FP64 mode: per tetrahedron edge n / l, m / l, t / l (n the normal, m, t the tangents,
+//                       l the length), d = l n, l A of its two facets, l, 2 l / (l_t - l); and
+//   grad   [3T][3] f64  grad N_i / 3 of the vertices 1..3, so that e_V = sum_i grad_i . (u_i - u_0): the
+//                       constants of the reference positions, which the FP64 pass would spend its pipe on
 //   fout   [12T]   R4   facet force acting on the edge's first vertex, 0 (written only when forces
 //                       are rebuilt from history, for ldpm_facet_forces)
 //   tvc    [T][4][6] R  per tetrahedron vertex: sum of its 6 facets' force (3) and moment about the
@@ -102,7 +106,8 @@ struct DeviceModel {
     int4 *tet = nullptr;
     void *geo = nullptr, *hist = nullptr, *fout = nullptr, *tvc = nullptr, *ent = nullptr;
     void *hist_out = nullptr;  // where a stepping facet pass writes the new history (null: hist, in place)
-    void *pf = nullptr;             // per-facet E0, alpha, sigma_t (R4 [12T]) or null
+    void *pf = nullptr;             // per-facet E0, alpha, sigma_t, 1 / alpha (R4 [12T]) or null
+    double *frame = nullptr, *grad = nullptr;  // FP64 mode: constants per edge and per tetrahedron
     int32_t *row = nullptr;
     int32_t *stab = nullptr;        // [N][kSlotTab] slot ids per particle (see the layout above)
     int32_t *tile_spec = nullptr;   // [T / tets_per_block] specimen of each tile, or null (all 0)
@@ -172,6 +177,8 @@ cudaError_t launch_persistent(const DeviceModel &m, int64_t nsteps, const Persis
 template <class R>
 cudaError_t launch_facet(const DeviceModel &m, int mode, const void *src_override, cudaStream_t s,
                          const BatchLaw *bl = nullptr);
+// FP64 mode: frame and grad of every tetrahedron from the positions, the arms and l_t.
+cudaError_t launch_frames(const DeviceModel &m, cudaStream_t s);
 // q += dq on free DOFs of the drifted state (dq [N][6] internal order, device), mirror updated.
 cudaError_t launch_perturb(const DeviceModel &m, const double *dq, cudaStream_t s);
 // Rebuild the FP32 mirror from pstate (after create, set_state, checkpoint load).  No-op in FP64.

@@ -3,12 +3,13 @@
 // One step (paper Sec. 3, central difference with lumped mass) is two launches.  Between steps the
 // state is kept drifted: q_{n+1} and v_{n+1/2} (and f_n); kick_kernel / unkick_kernel convert from /
 // to the whole-step state q_n, v_n at the API boundary.
-//   facet_kernel / facet_warp_kernel
+//   facet_kernel / facet_warp_kernel / facet_edge_kernel
 //                  per facet: rigid-body jump and strain (Sec. 2, Eq. (1)), per-tetrahedron
 //                  volumetric strain (App. A.2 e_V), the Appendix A law, force A P t; then per
 //                  tetrahedron vertex the fixed-order sum of its 6 facets' forces and moments
 //                  (the tetrahedron's share of Eq. (2a)-(2b)).  The warp variant (one 8-tetrahedron
-//                  tile per warp) runs the FP32 pass, the block variant the FP64 pass and larger tiles;
+//                  tile per warp) runs the FP32 pass, the edge variant (5 tetrahedra per warp, an edge per
+//                  lane) the FP64 step, the block variant the other FP64 passes and larger tiles;
 //   gather_kernel  per particle: fixed-order sum of its (tetrahedron, vertex) shares, then the second
 //                  half kick of this step, the energy increments, and the first half kick and drift
 //                  of the next step.
@@ -342,10 +343,8 @@ __device__ __forceinline__ void vertex_sum(const DeviceModel &m, int64_t tet0, i
 }
 
 // One tile of TETS tetrahedra run by a block of 12 TETS threads (one facet each): phases A-C above.
-// PF: the facet's own E0, alpha, sigma_t (m.pf) replace the material's in the law.  PERSIST: called
-// from the persistent step kernel (live data through ld_live; the block's shared rows are reused for
-// the next tile after the closing barrier).
-template <class R, int MODE, int TETS, bool PF, bool PERSIST>
+// PF: the facet's own E0, alpha, sigma_t (m.pf) replace the material's in the law.
+template <class R, int MODE, int TETS, bool PF>
 __device__ __forceinline__ void facet_block_tile(const DeviceModel &m, const void *__restrict__ vsrc, int64_t tet0,
                                                  R (*sv)[Stride<R>::row], R (*scon)[Stride<R>::con], R *seV,
                                                  int *sok)
@@ -364,12 +363,12 @@ __device__ __forceinline__ void facet_block_tile(const DeviceModel &m, const voi
     T4 g{}, h{}, pp{};
     if (valid) {
         g = geo[f];
-        if (MODE != FACET_ELASTIC) h = ld_live<PERSIST>(hist + f);
+        if (MODE != FACET_ELASTIC) h = hist[f];
         if (PF) pp = static_cast<const T4 *>(m.pf)[f];
     }
 
     // ---- phase A: vertex records -> shared memory, e_V per tetrahedron
-    if (tid < 4 * TETS) stage_vertex<R, MODE, PERSIST>(m, vsrc, tet0, tid, sv, seV, sok);
+    if (tid < 4 * TETS) stage_vertex<R, MODE>(m, vsrc, tet0, tid, sv, seV, sok);
     __syncthreads();
 
     // ---- phase B: one facet
@@ -382,7 +381,6 @@ __device__ __forceinline__ void facet_block_tile(const DeviceModel &m, const voi
 
     // ---- phase C
     if (live && MODE != FACET_METRIC) vertex_sum<R>(m, tet0, j, slot, scon);
-    if (PERSIST) __syncthreads();
 }
 
 template <class R, int MODE, int TETS, bool PF>
@@ -394,7 +392,7 @@ __global__ void __launch_bounds__(12 * TETS) facet_kernel(DeviceModel m, const v
     __shared__ int sok[TETS];
     const int64_t tet0 = (int64_t)blockIdx.x * TETS;
     if (MODE == FACET_STEP && blockIdx.x == 0 && threadIdx.x == 0) *m.step += 1;
-    facet_block_tile<R, MODE, TETS, PF, false>(m, vsrc, tet0, sv, scon, seV, sok);
+    facet_block_tile<R, MODE, TETS, PF>(m, vsrc, tet0, sv, scon, seV, sok);
 }
 
 // Warp-tile variant of facet_kernel: every warp owns a tile of 8 tetrahedra and runs phases A-C on it
@@ -536,6 +534,354 @@ __global__ void __launch_bounds__(32 * WPB, 12)
     if (MODE == FACET_STEP && blockIdx.x == 0 && threadIdx.x == 0) *m.step += 1;
     if (tet0 >= m.T) return;  // whole warp (T is a multiple of the tile)
     facet_tile<float, MODE, PF, false, false>(m, vsrc, tet0, lane, sv_[w], spl_[w], seV_[w], sok_[w], &bl.law[lo]);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Edge-tile facet pass of the FP64 step.  It is bound by the FP64 pipe (one warp instruction per ~64
+// cycles and sub-partition), so it is built to need few FP64 instructions; integer, FP32 and
+// shared-memory work is nearly free beside them.
+//   - A warp owns 5 tetrahedra and a lane one edge with its two facets (30 of 32 lanes): with
+//     d = x_b - x_a, [[u]] = (du - theta_b x d) + (theta_b - theta_a) x c, one cross product per edge
+//     and one per facet (c: the facet's arm from a) instead of two per facet; the moments about b are
+//     d x S - M_a with the two facets' S and M_a summed first.
+//   - The frame, the lengths and grad e_V depend on the reference positions alone and come from memory
+//     (m.frame, m.grad: 64 + 6 bytes per facet and step, 5 % of the pass at HBM rate).
+//   - Comparisons and the law's filters run on the other pipes (compression_trial64, fracture_floor32).
+//     The facets that may have reached a boundary are collected in shared memory, branch by branch, and
+//     evaluated by full warps (a tenth of them spread over a warp's 60 facets would otherwise hold all
+//     lanes twice).
+// Phases: records to shared memory with cp.async; one edge per lane; contributions vertex-major in three
+// planes (plane k: the k-th edge of each vertex), summed over the vertex's edges in ascending order.
+// Against the block kernel (one facet per thread, frames rebuilt, the whole law evaluated everywhere), per
+// launch on GB300 (ncu): 594 -> 225 us on 676k facets in tension past the peak, 540 -> 270 us on 1.15M
+// facets in compression; the FP64 pipe is 86 % busy in both.
+// ------------------------------------------------------------------------------------------------
+constexpr int kEdgeTets = 5;
+constexpr int kERow = 18;       // doubles per staged vertex record (16, padded against bank conflicts)
+constexpr int kEPlane = 122;    // doubles per contribution plane (20 vertices x 6 values, padded)
+constexpr int kEItem = 7;       // doubles per collected facet
+constexpr int kEWords = 12 * kEdgeTets * kEItem;  // doubles per warp; rows (360) and planes (366) lie in them
+static_assert(4 * kEdgeTets * kERow <= kEWords && 3 * kEPlane <= kEWords, "rows and planes fit");
+constexpr int kEdgeWarps = 2;   // warps (tiles) per block
+
+// 16-byte asynchronous copy into shared memory; zeros with `ok` false.  PERSIST: through L2 only.
+template <bool PERSIST>
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = ok ? 16 : 0;
+    if constexpr (PERSIST)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// Tetrahedra [tet0, tet0 + 5) by one warp on its own shared words sw (a tile may straddle two specimens:
+// the law constants are read per lane).
+template <bool PF, bool PERSIST>
+__device__ __forceinline__ void facet_edge_tile(const DeviceModel &m, const double *__restrict__ vsrc, int32_t tet0,
+                                                int lane, double *sw)
+{
+    const int j = lane / 6, e = lane - 6 * j, jj = j < kEdgeTets ? j : 0;
+    const int32_t tt = tet0 + j;
+    const bool in = lane < 6 * kEdgeTets && tt < m.T;
+    const double4a *__restrict__ geo = static_cast<const double4a *>(m.geo);
+    const double4a *hist = static_cast<const double4a *>(m.hist);
+    // ---- records to shared memory, this lane's facets to registers
+    int vid = -1;
+    if (lane < 4 * kEdgeTets && tet0 + (lane >> 2) < m.T)
+        vid = __ldg(reinterpret_cast<const int *>(m.tet) + 4 * (int64_t)tet0 + lane);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {  // 16-byte pieces 1..7 of each record (piece 0 is position only)
+        const int c = lane + 32 * i;
+        const int v = c / 7, part = 1 + c - 7 * v;
+        const int id = __shfl_sync(0xffffffffu, vid, v & 31);
+        if (c < 28 * kEdgeTets)
+            cp_async16<PERSIST>(sw + kERow * v + 2 * part, vsrc + (id >= 0 ? 16 * (int64_t)id + 2 * part : 0), id >= 0);
+    }
+    const bool live = __shfl_sync(0xffffffffu, vid, 4 * jj) >= 0 && in;
+    const int64_t f = 12 * (int64_t)tt + 2 * e;
+    double4a h[2] = {};
+    V3<double> P0{}, P1{}, P2{}, d{}, gr{};
+    double lA[2] = {}, ht = 0.0;
+    if (live) {
+        const double2 *fr = reinterpret_cast<const double2 *>(m.frame) + 8 * (6 * (int64_t)tt + e);
+        const double2 a0 = __ldg(fr), a1 = __ldg(fr + 1), a2 = __ldg(fr + 2), a3 = __ldg(fr + 3), a4 = __ldg(fr + 4),
+                      a5 = __ldg(fr + 5), a6 = __ldg(fr + 6), a7 = __ldg(fr + 7);
+        P0 = {a0.x, a0.y, a1.x};
+        P1 = {a1.y, a2.x, a2.y};
+        P2 = {a3.x, a3.y, a4.x};
+        d = {a4.y, a5.x, a5.y};
+        lA[0] = a6.x;
+        lA[1] = a6.y;
+        ht = a7.y;
+        if (e < 3) {
+            const double *g3 = m.grad + 3 * (3 * (int64_t)tt + e);
+            gr = {__ldg(g3), __ldg(g3 + 1), __ldg(g3 + 2)};
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) h[i] = ld_live<PERSIST>(hist + f + i);
+    }
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    // ---- one edge: local vertices va < vb
+    const int va = (0x211000 >> (4 * e)) & 0xF, vb = (0x332321 >> (4 * e)) & 0xF;
+    V3<double> wq, wv, dth, dom;
+    double eV;
+    {
+        // record: x 0..2, u 3..5, theta 6..8, v 9..11, omega 12..14
+        const double *A = sw + kERow * (4 * jj + va), *B = sw + kERow * (4 * jj + vb);
+        const V3<double> du = {B[3] - A[3], B[4] - A[4], B[5] - A[5]};
+        const V3<double> thB = {B[6], B[7], B[8]}, omB = {B[12], B[13], B[14]};
+        dth = {thB.x - A[6], thB.y - A[7], thB.z - A[8]};
+        dom = {omB.x - A[12], omB.y - A[13], omB.z - A[14]};
+        wv = add_cross(V3<double>{B[9] - A[9], B[10] - A[10], B[11] - A[11]}, d, omB);
+        wq = add_cross(du, d, thB);
+        // e_V: the edges 0-1, 0-2, 0-3 hold its three terms
+        const double term = fma(gr.x, du.x, fma(gr.y, du.y, gr.z * du.z));
+        const int base = 6 * jj;
+        const double t0 = __shfl_sync(0xffffffffu, term, base), t1 = __shfl_sync(0xffffffffu, term, base + 1),
+                     t2 = __shfl_sync(0xffffffffu, term, base + 2);
+        eV = t0 + t1 + t2;
+    }
+    __syncwarp();  // the rows are read: shared memory may be reused
+    const LawConst<double> &c = static_cast<const LawConst<double> *>(m.law)[in && m.tile_spec ? m.tile_spec[tt / 32] : 0];
+    V3<double> e3[2], t[2];  // strain; new traction (fracture: scalar effective traction in x until the end)
+    double emax[2], inv_e[2], aT2[2];
+    bool frac[2] = {false, false};
+    bool need[2] = {false, false};
+    auto par = [&](int i) -> FacetPar64 {
+        if constexpr (PF) {
+            const double4a pp = static_cast<const double4a *>(m.pf)[f + i];
+            return {pp.x, pp.y, pp.w, pp.z};
+        } else {
+            return {c.E0, c.alpha, c.inv_alpha, c.sigma_t};
+        }
+    };
+    if (live) {
+        const double dt = c.dt;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const double4a g = geo[f + i];
+            const V3<double> arm = {g.x, g.y, g.z};
+            const FacetPar64 fp = par(i);
+            const V3<double> J = add_cross(wq, dth, arm);
+            const V3<double> es = {fma(P0.x, J.x, fma(P0.y, J.y, P0.z * J.z)), fma(P1.x, J.x, fma(P1.y, J.y, P1.z * J.z)),
+                                   fma(P2.x, J.x, fma(P2.y, J.y, P2.z * J.z))};
+            e3[i] = es;
+            emax[i] = h[i].w;
+            if (c.elastic) {
+                const double aE = fp.alpha * fp.E0;
+                t[i] = {fp.E0 * es.x, aE * es.y, aE * es.z};
+                continue;
+            }
+            const V3<double> Jv = add_cross(wv, dom, arm);
+            const V3<double> de = {dt * fma(P0.x, Jv.x, fma(P0.y, Jv.y, P0.z * Jv.z)),
+                                   dt * fma(P1.x, Jv.x, fma(P1.y, Jv.y, P1.z * Jv.z)),
+                                   dt * fma(P2.x, Jv.x, fma(P2.y, Jv.y, P2.z * Jv.z))};
+            const double tN = h[i].x, tM = h[i].y, tL = h[i].z;
+            if (order_bits(es.x) <= 0) {
+                t[i] = {tN, tM, tL};
+                need[i] = compression_trial64(c, fp, de, t[i]);
+                continue;
+            }
+            // fracture (App. A.1), as facet_law; e = e^2 / e from the reciprocal root
+            const double a2 = fp.alpha * fma(es.y, es.y, es.z * es.z);
+            const double e2 = fma(es.x, es.x, a2);
+            if (order_bits(e2) < order_bits(1e-300)) {  // e < c.tiny_strain = 1e-150: t = E e
+                const double aE = fp.alpha * fp.E0, eff = sqrt(e2);
+                t[i] = {fp.E0 * es.x, aE * es.y, aE * es.z};
+                emax[i] = order_bits(emax[i]) > order_bits(eff) ? emax[i] : eff;
+                continue;
+            }
+            frac[i] = true;
+            const double ie = rsqrt(e2), eff = e2 * ie;
+            const double em = order_bits(emax[i]) > order_bits(eff) ? emax[i] : eff;
+            const V3<double> ep = es - de;
+            const double e_old = sqrt(fma(ep.x, ep.x, fp.alpha * fma(ep.y, ep.y, ep.z * ep.z)));
+            const double num = fma(de.x, es.x + ep.x, fp.alpha * fma(de.y, es.y + ep.y, de.z * (es.z + ep.z)));
+            double d_eff = num / (eff + e_old);
+            const double t_old = sqrt(fma(tN, tN, fma(tM, tM, tL * tL) * fp.inv_alpha));
+            if (c.k_t > 0.0 && t_old <= 0.0 && d_eff > 0.0) {
+                // reloading from zero traction: it stays zero up to e_tr = k_t (e_max - sigma_bt / E0)
+                const double e_tr = c.k_t * (em - fracture_boundary64(c, fp, es.x, a2, ie, em, ht) / fp.E0);
+                if (e_tr > e_old) d_eff = eff > e_tr ? eff - e_tr : 0.0;
+            }
+            double tr = fma(fp.E0, d_eff, t_old);
+            tr = order_bits(tr) < 0 ? 0.0 : tr;
+            const float E0f = d2f_trunc(fp.E0), stf = d2f_trunc(fp.sigma_t), trf = d2f_trunc(tr), emf = d2f_trunc(em);
+            const float k4 = d2f_trunc(fp.alpha) * d2f_trunc(c.four_over_r2);
+            // sigma_0 >= 2 sigma_t / (1 + sqrt(max(1, 4 alpha / r_st^2))) for every omega
+            const float s0min = 0.9999f * 2.0f * stf / (1.0f + sqrtf(fmaxf(1.0f, k4)));
+            need[i] = !(E0f * emf <= s0min && trf <= s0min) &&
+                      !(trf <= fracture_floor32(E0f, k4, d2f_trunc(c.r_s) * E0f / d2f_trunc(fp.alpha), stf,
+                                                d2f_trunc(c.n_t), d2f_trunc(es.x), d2f_trunc(a2), d2f_trunc(ie), emf,
+                                                d2f_trunc(ht)) * 0.9999f);
+            t[i].x = tr;
+            emax[i] = em;
+            inv_e[i] = ie;
+            aT2[i] = a2;
+        }
+    }
+    // ---- the facets that may have reached a boundary, collected per branch: item k goes to lane k % 32
+    const int sp = m.tile_spec && in ? m.tile_spec[tt / 32] : 0;
+#pragma unroll
+    for (int br = 0; br < 2; ++br) {  // 0: fracture, 1: compression and friction
+        const bool n0 = need[0] && frac[0] == (br == 0), n1 = need[1] && frac[1] == (br == 0);
+        const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
+        const int items = __popc(b0) + __popc(b1);
+        if (!items) continue;
+        const unsigned below = (1u << lane) - 1u;
+        double *w0 = sw + kEItem * __popc(b0 & below), *w1 = sw + kEItem * (__popc(b0) + __popc(b1 & below));
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (i == 0 ? n0 : n1) {
+                double *w = i == 0 ? w0 : w1;
+                w[0] = t[i].x;
+                w[1] = e3[i].x;
+                w[2] = br == 0 ? aT2[i] : t[i].y;
+                w[3] = br == 0 ? inv_e[i] : t[i].z;
+                w[4] = br == 0 ? emax[i] : eV;
+                if (br == 0) w[5] = ht;
+                w[6] = __longlong_as_double((f + i) | ((long long)sp << 40));
+            }
+        __syncwarp();
+        for (int k = lane; k < items; k += 32) {
+            double *w = sw + kEItem * k;
+            const long long id = __double_as_longlong(w[6]);
+            const LawConst<double> &ck = static_cast<const LawConst<double> *>(m.law)[id >> 40];
+            FacetPar64 fp = {ck.E0, ck.alpha, ck.inv_alpha, ck.sigma_t};
+            if constexpr (PF) {
+                const double4a pp = static_cast<const double4a *>(m.pf)[id & 0xffffffffffll];
+                fp = {pp.x, pp.y, pp.w, pp.z};
+            }
+            if (br == 0) {
+                const double sb = fracture_boundary64(ck, fp, w[1], w[2], w[3], w[4], w[5]);
+                if (order_bits(w[0]) > order_bits(sb)) w[0] = sb;
+            } else {
+                V3<double> tr = {w[0], w[2], w[3]};
+                compression_return64(ck, fp, w[1], w[4], tr);
+                w[0] = tr.x;
+                w[2] = tr.y;
+                w[3] = tr.z;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (i == 0 ? n0 : n1) {
+                const double *w = i == 0 ? w0 : w1;
+                t[i].x = w[0];
+                if (br == 1) {
+                    t[i].y = w[2];
+                    t[i].z = w[3];
+                }
+            }
+        __syncwarp();
+    }
+    if (live) {
+        double4a *__restrict__ hout = static_cast<double4a *>(m.hist_out ? m.hist_out : m.hist);
+        V3<double> S{}, MA{};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (frac[i]) {
+                const double r = t[i].x * inv_e[i], ar = par(i).alpha * r;
+                t[i] = {r * e3[i].x, ar * e3[i].y, ar * e3[i].z};
+            }
+            double4a hn;
+            hn.x = t[i].x;
+            hn.y = t[i].y;
+            hn.z = t[i].z;
+            hn.w = emax[i];
+            hout[f + i] = hn;
+            const double4a g = geo[f + i];
+            const V3<double> a = lA[i] * t[i];
+            const V3<double> F = {fma(a.x, P0.x, fma(a.y, P1.x, a.z * P2.x)), fma(a.x, P0.y, fma(a.y, P1.y, a.z * P2.y)),
+                                  fma(a.x, P0.z, fma(a.y, P1.z, a.z * P2.z))};
+            S = S + F;
+            MA = add_cross(MA, V3<double>{g.x, g.y, g.z}, F);
+        }
+        // end a receives (S, MA), end b (-S, d x S - MA); e is the ka-th edge of va, the kb-th of vb
+        const int ka = (0x221210 >> (4 * e)) & 0xF, kb = (0x211000 >> (4 * e)) & 0xF;
+        const V3<double> MB = add_cross(V3<double>{-MA.x, -MA.y, -MA.z}, d, S);
+        double2 *da = reinterpret_cast<double2 *>(sw + ka * kEPlane + 6 * (4 * j + va));
+        double2 *db = reinterpret_cast<double2 *>(sw + kb * kEPlane + 6 * (4 * j + vb));
+        da[0] = double2{S.x, S.y};
+        da[1] = double2{S.z, MA.x};
+        da[2] = double2{MA.y, MA.z};
+        db[0] = double2{-S.x, -S.y};
+        db[1] = double2{-S.z, MB.x};
+        db[2] = double2{MB.y, MB.z};
+    }
+    const unsigned lv = __ballot_sync(0xffffffffu, live);
+    __syncwarp();
+    // ---- pair q of the tile's 120 share values over the vertex's three edges
+    double2 *__restrict__ out = reinterpret_cast<double2 *>(static_cast<double *>(m.tvc) + 24 * (int64_t)tet0);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int q = lane + 30 * i;
+        if (lane < 30 && ((lv >> (6 * (q / 12))) & 1u)) {
+            const double2 *s2 = reinterpret_cast<const double2 *>(sw) + q;
+            const double2 x = s2[0], y = s2[kEPlane / 2], z = s2[kEPlane];
+            out[q] = double2{(x.x + y.x) + z.x, (x.y + y.y) + z.y};
+        }
+    }
+    if (PERSIST) __syncwarp();  // the shared words are reused for the next tile
+}
+
+template <bool PF>
+__global__ void __launch_bounds__(32 * kEdgeWarps)
+    facet_edge_kernel(const __grid_constant__ DeviceModel m, const double *__restrict__ vsrc)
+{
+    __shared__ alignas(16) double sw[kEdgeWarps][kEWords];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t tet0 = ((int64_t)blockIdx.x * kEdgeWarps + w) * kEdgeTets;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *m.step += 1;
+    if (tet0 >= m.T) return;  // the whole warp
+    facet_edge_tile<PF, false>(m, vsrc, (int32_t)tet0, lane, sw[w]);
+}
+
+// m.frame and m.grad (see ldpm_internal.h) from the reference positions; one thread per edge.
+__global__ void __launch_bounds__(128) frame_kernel(DeviceModel m)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= 6 * (int64_t)m.T) return;
+    const int64_t tt = k / 6;
+    const int e = (int)(k - 6 * tt);
+    double *fr = m.frame + 16 * k;
+    const int *tv = reinterpret_cast<const int *>(m.tet) + 4 * tt;
+    if (tv[0] < 0) {
+        for (int q = 0; q < 16; ++q) fr[q] = 0.0;
+        if (e < 3)
+            for (int q = 0; q < 3; ++q) m.grad[3 * (3 * tt + e) + q] = 0.0;
+        return;
+    }
+    V3<double> x[4];
+    for (int v = 0; v < 4; ++v) {
+        const double *p = m.pstate + 16 * (int64_t)tv[v];
+        x[v] = {p[0], p[1], p[2]};
+    }
+    const int va = (0x211000 >> (4 * e)) & 0xF, vb = (0x332321 >> (4 * e)) & 0xF;
+    const V3<double> d = x[vb] - x[va];
+    const double l2 = dot(d, d), l = sqrt(l2), il = 1.0 / l;
+    const V3<double> n = il * d;
+    V3<double> mt, lt;
+    tangent_frame(n, mt, lt);
+    const double lim = static_cast<const LawConst<double> *>(m.law)[m.tile_spec ? m.tile_spec[tt / 32] : 0].l_t;
+    const double4a *geo = static_cast<const double4a *>(m.geo) + 2 * k;
+    const double rec[16] = {il * n.x, il * n.y, il * n.z, il * mt.x, il * mt.y, il * mt.z, il * lt.x, il * lt.y,
+                            il * lt.z, d.x, d.y, d.z, l * geo[0].w, l * geo[1].w, l, 2.0 * l / (lim - l)};
+    for (int q = 0; q < 16; ++q) fr[q] = rec[q];
+    if (e < 3) {
+        const V3<double> dx[3] = {x[1] - x[0], x[2] - x[0], x[3] - x[0]};
+        const double det = dot(dx[0], cross(dx[1], dx[2]));
+        const V3<double> g = cross(dx[(e + 1) % 3], dx[(e + 2) % 3]);
+        const double s = det != 0.0 ? 1.0 / (3.0 * det) : 0.0;
+        double *o = m.grad + 3 * (3 * tt + e);
+        o[0] = s * g.x;
+        o[1] = s * g.y;
+        o[2] = s * g.z;
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -892,36 +1238,30 @@ __global__ void __launch_bounds__(32 * WPB)
     }
 }
 
-// FP64 variant: the facet phase takes 8-tetrahedron tiles per block of 96 threads, one facet per thread
-// (facet_block_tile, as facet_kernel does), which gives the FP64 pipe 4x the warps of warp tiles with
-// three facets per lane.  The particle phase is the warp-level one of the kernel above.
-template <class R, bool PF>
-__global__ void __launch_bounds__(12 * kTileTets)
-    step_persistent_block_kernel(const __grid_constant__ DeviceModel m, const void *__restrict__ vsrc, int64_t nsteps,
-                                 PersistCtl ctl)
+// FP64 variant: the facet phase takes the edge tiles of facet_edge_kernel.
+template <bool PF, int WPB>
+__global__ void __launch_bounds__(32 * WPB)
+    step_persistent_edge_kernel(const __grid_constant__ DeviceModel m, const double *__restrict__ vsrc, int64_t nsteps,
+                                PersistCtl ctl)
 {
-    constexpr int TETS = kTileTets;
-    constexpr int WPB = 12 * TETS / 32;
-    __shared__ alignas(16) R sv[TETS * 4][Stride<R>::row];
-    __shared__ alignas(16) R scon[12 * TETS][Stride<R>::con];
-    __shared__ R seV[TETS];
-    __shared__ int sok[TETS];
+    __shared__ alignas(16) double sw[WPB][kEWords];
     __shared__ int s_stop;
     if (threadIdx.x == 0) s_stop = *(volatile const int32_t *)ctl.status;
     __syncthreads();
     if (s_stop != 0) return;  // an earlier launch gave up: no work (the whole block)
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)blockIdx.x * WPB + w, nw = (int64_t)gridDim.x * WPB;
-    const int64_t tiles = m.T / TETS;
+    const int64_t tiles = ((int64_t)m.T + kEdgeTets - 1) / kEdgeTets;
     const int64_t groups = ((int64_t)m.N + 3) / 4;
     unsigned target = 0;
     for (int64_t n = 0; n < nsteps; ++n) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *m.step += 1;
-        for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x)
-            facet_block_tile<R, FACET_STEP, TETS, PF, true>(m, vsrc, t * TETS, sv, scon, seV, sok);
+        for (int64_t t = gw; t < tiles; t += nw)
+            facet_edge_tile<PF, true>(m, vsrc, (int32_t)(t * kEdgeTets), lane, sw[w]);
         target += gridDim.x;
         if (!grid_barrier(ctl, target, !(n == 0 && (int)blockIdx.x == ctl.skip_block))) return;
-        for (int64_t g = gw; g < groups; g += nw) gather_group<R, GATHER_STEP_MID, 8, true>(m, 4 * g + lane / 8, lane, nullptr);
+        for (int64_t g = gw; g < groups; g += nw)
+            gather_group<double, GATHER_STEP_MID, 8, true>(m, 4 * g + lane / 8, lane, nullptr);
         target += gridDim.x;
         if (!grid_barrier(ctl, target, true)) return;
     }
@@ -930,7 +1270,7 @@ __global__ void __launch_bounds__(12 * kTileTets)
 template <class R, bool PF, bool S1>
 constexpr int persist_wpb()
 {
-    return sizeof(R) == 4 ? 4 : 12 * kTileTets / 32;  // static shared memory stays below 48 KB per block
+    return sizeof(R) == 4 ? 4 : 2;  // static shared memory stays below 48 KB per block
 }
 
 template <class R, bool PF, bool S1>
@@ -939,7 +1279,7 @@ const void *persist_fn()
     if constexpr (sizeof(R) == 4)
         return reinterpret_cast<const void *>(&step_persistent_kernel<R, PF, S1, persist_wpb<R, PF, S1>()>);
     else
-        return reinterpret_cast<const void *>(&step_persistent_block_kernel<R, PF>);
+        return reinterpret_cast<const void *>(&step_persistent_edge_kernel<PF, persist_wpb<R, PF, S1>()>);
 }
 
 // First half kick and drift of a stepping call: v_{n+1/2} = v_n + dt/2 a_n, q_{n+1} = q_n + dt v_{n+1/2}.
@@ -1222,19 +1562,29 @@ cudaError_t launch_facet_pf(const DeviceModel &m, const void *pst, cudaStream_t 
     const unsigned blocks = (unsigned)((m.T + tpb - 1) / tpb);
     if (blocks == 0) return cudaSuccess;
     // FP32 facet pass with 8-tetrahedron tiles: one tile per warp, 2 warps per block (measured on GB300:
-    // 43.6 us against 47.4 us for the 96-thread block kernel on 1.82M facets).  The FP64 pass, bound by
-    // the FP64 pipe, is 4 % faster with the block kernel.
-    if (sizeof(R) == 4 && tpb == kTileTets) {
-        constexpr int WPB = 2;
-        const int64_t tiles = (m.T + kTileTets - 1) / kTileTets;
-        const unsigned nb = (unsigned)((tiles + WPB - 1) / WPB);
-        if (m.n_spec == 1)
-            facet_warp_kernel<R, MODE, WPB, PF, true><<<nb, 32 * WPB, 0, s>>>(m, pst);
-        else if (bl && bl->n == m.n_spec)
-            facet_warp_batch_kernel<MODE, WPB, PF><<<nb, 32 * WPB, 0, s>>>(m, pst, *bl);
-        else
-            facet_warp_kernel<R, MODE, WPB, PF, false><<<nb, 32 * WPB, 0, s>>>(m, pst);
-        return cudaGetLastError();
+    // 43.6 us against 47.4 us for the 96-thread block kernel on 1.82M facets).
+    if constexpr (sizeof(R) == 4) {
+        if (tpb == kTileTets) {
+            constexpr int WPB = 2;
+            const int64_t tiles = (m.T + kTileTets - 1) / kTileTets;
+            const unsigned nb = (unsigned)((tiles + WPB - 1) / WPB);
+            if (m.n_spec == 1)
+                facet_warp_kernel<R, MODE, WPB, PF, true><<<nb, 32 * WPB, 0, s>>>(m, pst);
+            else if (bl && bl->n == m.n_spec)
+                facet_warp_batch_kernel<MODE, WPB, PF><<<nb, 32 * WPB, 0, s>>>(m, pst, *bl);
+            else
+                facet_warp_kernel<R, MODE, WPB, PF, false><<<nb, 32 * WPB, 0, s>>>(m, pst);
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (sizeof(R) == 8 && MODE == FACET_STEP) {
+        // the FP64 step: edge tiles, unless a launch shape of 16 or 32 tetrahedra per block was asked for
+        if (tpb == 8) {
+            const int64_t tiles = (m.T + kEdgeTets - 1) / kEdgeTets;
+            facet_edge_kernel<PF><<<(unsigned)((tiles + kEdgeWarps - 1) / kEdgeWarps), 32 * kEdgeWarps, 0, s>>>(
+                m, static_cast<const double *>(pst));
+            return cudaGetLastError();
+        }
     }
     switch (tpb) {
     case 16:
@@ -1276,11 +1626,11 @@ cudaError_t launch_persistent_r(const DeviceModel &m, int64_t nsteps, const Pers
     if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
     // as many blocks as the device holds at once, but no more than the work needs: every block takes
     // part in every barrier, so idle blocks on a small specimen would only slow the barriers down
-    // (a tile takes a warp in the FP32 kernel and a block in the FP64 one; 4 particles take a warp)
+    // (a tile takes a warp, as do 4 particles)
     const int wpb = threads / 32;
-    const int64_t tiles = m.T / kTileTets, groups = ((int64_t)m.N + 3) / 4;
-    const int64_t need = sizeof(R) == 4 ? (std::max(tiles, groups) + wpb - 1) / wpb
-                                        : std::max(tiles, (groups + wpb - 1) / wpb);
+    constexpr int tets = sizeof(R) == 4 ? kTileTets : kEdgeTets;
+    const int64_t tiles = ((int64_t)m.T + tets - 1) / tets, groups = ((int64_t)m.N + 3) / 4;
+    const int64_t need = (std::max(tiles, groups) + wpb - 1) / wpb;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * sms, need));
     if (grid_out) *grid_out = (int)grid;
     if (nsteps <= 0) return cudaSuccess;
@@ -1369,6 +1719,14 @@ cudaError_t launch_gather(const DeviceModel &m, int mode, double *out6, cudaStre
     default:
         return launch_gather_lpp<R, 8>(m, mode, out6, s);
     }
+}
+
+cudaError_t launch_frames(const DeviceModel &m, cudaStream_t s)
+{
+    const int64_t n = 6 * (int64_t)m.T;
+    if (!m.frame || n == 0) return cudaSuccess;
+    frame_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(m);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mirror(const DeviceModel &m, cudaStream_t s)
