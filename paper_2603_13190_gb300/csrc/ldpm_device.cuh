@@ -416,6 +416,21 @@ __device__ __forceinline__ double f2d_bits(float f)
     return __longlong_as_double((long long)(sign | (ed << 52) | ((uint64_t)(u & 0x7fffffu) << 29)));
 }
 
+// a * b as a double, exactly (48 mantissa bits), with integer instructions; subnormal operands count as
+// zero, as everywhere in these translation units.
+__device__ __forceinline__ double mul_exact(float a, float b)
+{
+    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+    const uint32_t ea = (ua >> 23) & 0xffu, eb = (ub >> 23) & 0xffu;
+    const uint64_t sign = (uint64_t)((ua ^ ub) & 0x80000000u) << 32;
+    if (ea == 255 || eb == 255) return f2d_bits(a * b);  // an infinity or NaN, with FP32's class
+    if (ea == 0 || eb == 0) return __longlong_as_double((long long)sign);
+    const uint64_t p = (uint64_t)((ua & 0x7fffffu) | 0x800000u) * ((ub & 0x7fffffu) | 0x800000u);
+    const int top = (int)(p >> 47);  // the product of two mantissas in [1, 2) is in [1, 4)
+    return __longlong_as_double(
+        (long long)(sign | ((uint64_t)(ea + eb + 769 + top) << 52) | ((p << (6 - top)) & 0xfffffffffffffull)));
+}
+
 // ------------------------------------------------------------------------------------------------
 // Compensated ("float-float") arithmetic on the FP32 pipe.  A value is the unevaluated sum hi + lo of
 // two floats (48 mantissa bits).  two_sum is Knuth's error-free addition (TAOCP vol. 2, 4.2.2):

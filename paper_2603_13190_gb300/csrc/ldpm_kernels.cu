@@ -1514,27 +1514,57 @@ __device__ __forceinline__ bool facet_frame_of(const DeviceModel &m, int64_t f, 
 
 // History of n facets in the caller's order: umap[k] = 2 f + s for internal facet f, s = 1 where the
 // caller's facet runs from the internal vertex b to a (the tangential traction vector flips sign).
+// The FP64 pipe (conversions included) bound this read-out: mixed mode now forms the products of two
+// floats exactly with integer instructions and spends one FP64 addition per component (the same bits as
+// FP64 arithmetic gives), FP64 mode takes the stored frames.  The 5 values per facet go through shared
+// memory so that a block writes one contiguous range.  11.4M facets, mixed: 401 -> 180 us; 1.15M
+// facets, FP64: 99 -> 27 us (ncu).
+constexpr int kHistBlock = 128;
 template <class R>
-__global__ void hist_to_user_kernel(DeviceModel m, const int32_t *__restrict__ umap, int64_t nf,
-                                    double *__restrict__ out5)
+__global__ void __launch_bounds__(kHistBlock)
+    hist_to_user_kernel(DeviceModel m, const int32_t *__restrict__ umap, int64_t nf, double *__restrict__ out5)
 {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nf) return;
-    const int32_t code = umap[k];
-    const int64_t f = code >> 1;
-    const double sg = (code & 1) ? -1.0 : 1.0;
-    V3<R> n, mt, lt;
-    const R4<R> h = static_cast<const R4<R> *>(m.hist)[f];
-    double *o = out5 + 5 * k;
-    if (!facet_frame_of<R>(m, f, n, mt, lt)) {
-        for (int c = 0; c < 5; ++c) o[c] = 0.0;
-        return;
+    __shared__ double s5[5 * kHistBlock];
+    const int64_t k0 = (int64_t)blockIdx.x * kHistBlock, k = k0 + threadIdx.x;
+    if (k < nf) {
+        const int32_t code = umap[k];
+        const int64_t f = code >> 1;
+        const R4<R> h = static_cast<const R4<R> *>(m.hist)[f];
+        double o[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        if constexpr (sizeof(R) == 4) {
+            V3<float> n, mt, lt;
+            if (facet_frame_of<float>(m, f, n, mt, lt)) {
+                o[0] = f2d_bits(h.x);
+                o[1] = mul_exact(h.y, mt.x) + mul_exact(h.z, lt.x);
+                o[2] = mul_exact(h.y, mt.y) + mul_exact(h.z, lt.y);
+                o[3] = mul_exact(h.y, mt.z) + mul_exact(h.z, lt.z);
+                o[4] = f2d_bits(h.w);
+            }
+        } else {
+            const int64_t ed = f >> 1;  // the facet's edge: m / l at 3..5, t / l at 6..8, l at 14 of its frame
+            const double *fr = m.frame + 16 * ed;
+            if (fr[14] > 0.0) {
+                const double a = h.y * fr[14], b = h.z * fr[14];
+                o[0] = h.x;
+                o[1] = fma(a, fr[3], b * fr[6]);
+                o[2] = fma(a, fr[4], b * fr[7]);
+                o[3] = fma(a, fr[5], b * fr[8]);
+                o[4] = h.w;
+            }
+        }
+        const long long flip = (long long)(code & 1) << 63;
+#pragma unroll
+        for (int c = 0; c < 5; ++c)
+            s5[5 * threadIdx.x + c] =
+                c >= 1 && c <= 3 ? __longlong_as_double(__double_as_longlong(o[c]) ^ flip) : o[c];
     }
-    o[0] = double(h.x);
-    o[1] = sg * (double(h.y) * double(mt.x) + double(h.z) * double(lt.x));
-    o[2] = sg * (double(h.y) * double(mt.y) + double(h.z) * double(lt.y));
-    o[3] = sg * (double(h.y) * double(mt.z) + double(h.z) * double(lt.z));
-    o[4] = double(h.w);
+    __syncthreads();
+    const int64_t n5 = 5 * (nf - k0 < kHistBlock ? nf - k0 : (int64_t)kHistBlock);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        const int i = threadIdx.x + c * kHistBlock;
+        if (i < n5) out5[5 * k0 + i] = s5[i];
+    }
 }
 
 template <class R>
@@ -1757,7 +1787,7 @@ template <class R>
 cudaError_t launch_hist_to_user(const DeviceModel &m, const int32_t *umap, int64_t n, double *out5, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    hist_to_user_kernel<R><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(m, umap, n, out5);
+    hist_to_user_kernel<R><<<(unsigned)((n + kHistBlock - 1) / kHistBlock), kHistBlock, 0, s>>>(m, umap, n, out5);
     return cudaGetLastError();
 }
 
