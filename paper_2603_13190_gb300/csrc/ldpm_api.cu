@@ -210,7 +210,7 @@ struct ldpm_ctx {
     std::vector<double> x_int;     // [N][3] internal order
     std::vector<double> inv_mass;  // [N][6]
     std::vector<double> pconst_h;  // [N][8]
-    double *d_partial = nullptr, *d_out16 = nullptr, *h_out16 = nullptr;
+    double *d_partial = nullptr, *h_out18 = nullptr;  // energy read-back: block sums; pinned result
     unsigned *d_ticket = nullptr;       // block counter of the energy reduction
     int32_t *d_umap = nullptr;          // caller's facets of all specimens, concatenated: 2 f + orientation flip
     int32_t *d_pmap = nullptr;          // caller's particles of all specimens, concatenated: internal particle
@@ -242,11 +242,11 @@ void free_model(ldpm_ctx *h)
                     h->dm.tet,
                     h->dm.geo,
                     h->dm.hist, h->dm.fout, h->dm.tvc, h->dm.ent, h->dm.row, h->dm.stab, h->dm.tile_spec, h->dm.law, h->dm.spec,
-                    h->dm.step, h->dm.flag, h->d_partial, h->d_out16, h->dm.pf, h->d_umap, h->d_scratch, h->d_ticket,
+                    h->dm.step, h->dm.flag, h->d_partial, h->dm.pf, h->d_umap, h->d_scratch, h->d_ticket,
                     h->d_pmap, h->pctl.arrive, h->pctl.status, h->dm.frame, h->dm.grad};
     for (void *p : ptrs)
         if (p) cudaFree(p);
-    if (h->h_out16) cudaFreeHost(h->h_out16);
+    if (h->h_out18) cudaFreeHost(h->h_out18);
     for (auto e : h->ev_pool) cudaEventDestroy(e);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
@@ -976,8 +976,8 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
         (rc = dalloc(&dm.tet, (size_t)T)) || (rc = dalloc(&dm.row, (size_t)N + 1)) ||
         (rc = dalloc(&dm.stab, (size_t)kSlotTab * N)) ||
         (rc = dalloc(&dm.tile_spec, (size_t)T / kTile)) || (rc = dalloc(&dm.spec, (size_t)n)) ||
-        (rc = dalloc(&dm.step, 1)) || (rc = dalloc(&dm.flag, 1)) || (rc = dalloc(&h->d_out16, 16)) ||
-        (rc = dalloc(&h->d_partial, 16 * (size_t)((N + 255) / 256 + 1))) || (rc = dalloc(&h->d_umap, umap.size())) ||
+        (rc = dalloc(&dm.step, 1)) || (rc = dalloc(&dm.flag, 1)) || (rc = dalloc(&h->d_partial, kEnergyPartials)) ||
+        (rc = dalloc(&h->d_umap, umap.size())) ||
         (rc = dalloc(&h->d_ticket, 1)) || (rc = dalloc(&h->d_pmap, (size_t)N)) ||
         (rc = dalloc(&h->pctl.arrive, 1)) || (rc = dalloc(&h->pctl.status, 1)))
         return rc;
@@ -999,7 +999,7 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
         CU(cudaMemcpy(dm.f_ext, H.f_ext.data(), H.f_ext.size() * sizeof(double), cudaMemcpyHostToDevice));
     }
     if (h->prec == LDPM_MIXED && (rc = dalloc(&dm.pm32, (size_t)kMirror * N))) return rc;
-    CU(cudaMallocHost((void **)&h->h_out16, 16 * sizeof(double)));
+    CU(cudaMallocHost((void **)&h->h_out18, 18 * sizeof(double)));
     CU(cudaMemcpy(dm.pstate, H.pstate.data(), H.pstate.size() * sizeof(double), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dm.pdyn, H.pdyn.data(), H.pdyn.size() * sizeof(double), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double), cudaMemcpyHostToDevice));
@@ -1221,18 +1221,24 @@ int timed(ldpm_ctx *h, int kid, Fn &&launch)
     return LDPM_OK;
 }
 
-int check_flag(ldpm_ctx *h)
+// The error a non-finite flag or a barrier status stands for.
+int flag_result(ldpm_ctx *h, int32_t fl, int32_t st)
 {
-    int32_t fl = 0, st = 0;
-    CU(cudaMemcpyAsync(&fl, h->dm.flag, sizeof(fl), cudaMemcpyDeviceToHost, h->stream));
-    CU(cudaMemcpyAsync(&st, h->pctl.status, sizeof(st), cudaMemcpyDeviceToHost, h->stream));
-    CU(cudaStreamSynchronize(h->stream));
     if (st)
         return fail(LDPM_E_TIMEOUT, "a grid barrier of the persistent step kernel waited longer than %.3g s; the "
                     "state is undefined until ldpm_set_state or ldpm_load_checkpoint",
                     1e-9 * (double)h->pctl.wait_ns);
     if (fl) return fail(LDPM_E_UNSTABLE, "non-finite velocity or displacement (time step too large?)");
     return LDPM_OK;
+}
+
+int check_flag(ldpm_ctx *h)
+{
+    int32_t fl = 0, st = 0;
+    CU(cudaMemcpyAsync(&fl, h->dm.flag, sizeof(fl), cudaMemcpyDeviceToHost, h->stream));
+    CU(cudaMemcpyAsync(&st, h->pctl.status, sizeof(st), cudaMemcpyDeviceToHost, h->stream));
+    CU(cudaStreamSynchronize(h->stream));
+    return flag_result(h, fl, st);
 }
 
 struct DevGuard {
@@ -1675,11 +1681,11 @@ int ldpm_set_state(ldpm_t h, const double *q, const double *v, const double *his
 static int energy_of(ldpm_t h, int s, double out[4], double reaction[12])
 {
     const SpecHost &S = h->sp[s];
-    cudaError_t e = launch_energy(h->dm, S.p0, S.p0 + S.N, h->d_partial, h->d_ticket, h->d_out16, h->stream);
+    // one kernel and one wait: it writes the sums and the handle's error words to pinned host memory
+    cudaError_t e = launch_energy(h->dm, S.p0, S.p0 + S.N, h->d_partial, h->d_ticket, h->pctl.status, h->h_out18, h->stream);
     if (e != cudaSuccess) return fail(LDPM_E_CUDA, "energy launch: %s", cudaGetErrorString(e));
-    CU(cudaMemcpyAsync(h->h_out16, h->d_out16, 16 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CU(cudaStreamSynchronize(h->stream));
-    const double *r = h->h_out16;
+    const double *r = h->h_out18;
     const double Wint = r[0], Wext = r[1], Wkin = r[2];
     if (out) {
         out[0] = Wext;
@@ -1690,7 +1696,7 @@ static int energy_of(ldpm_t h, int s, double out[4], double reaction[12])
     }
     if (reaction)
         for (int k = 0; k < 12; ++k) reaction[k] = r[4 + k];
-    return LDPM_OK;
+    return flag_result(h, (int)r[16], (int)r[17]);
 }
 
 int ldpm_energy(ldpm_t h, double out[4], double reaction[12])
@@ -1699,9 +1705,7 @@ int ldpm_energy(ldpm_t h, double out[4], double reaction[12])
     if (!h || !out) return fail(LDPM_E_INVALID_ARG, "bad handle or NULL out");
     if (h->sp.size() != 1) return fail(LDPM_E_INVALID_ARG, "batch handle: use ldpm_batch_energy");
     DevGuard dg(h->device);
-    int rc = energy_of(h, 0, out, reaction);
-    if (rc) return rc;
-    return check_flag(h);
+    return energy_of(h, 0, out, reaction);
 }
 
 int ldpm_facet_forces(ldpm_t h, double *F3, double *f6)
@@ -1968,9 +1972,7 @@ int ldpm_batch_energy(ldpm_t h, int32_t idx, double out[4], double reaction[12])
     if (!h || !out || idx < 0 || idx >= (int32_t)h->sp.size())
         return fail(LDPM_E_INVALID_ARG, "bad handle, index or NULL out");
     DevGuard dg(h->device);
-    int rc = energy_of(h, idx, out, reaction);
-    if (rc) return rc;
-    return check_flag(h);
+    return energy_of(h, idx, out, reaction);
 }
 
 int ldpm_batch_metrics(ldpm_t h, int32_t idx, double *crack_opening, double *tet_volumetric_strain)

@@ -1396,86 +1396,106 @@ __global__ void __launch_bounds__(256) perturb_kernel(DeviceModel m, const doubl
     if (m.pm32) write_mirror(m.pm32 + kMirror * p, d, q, ps[9 + d]);
 }
 
-// Energy sums over particles [p0, p1) (per block, fixed order), then one block adds the partials.
-// Warp sum of 16 values per lane by halving exchanges: at each level a lane keeps half of its values
-// and adds its partner's copy of that half (8 + 4 + 2 + 1 + 1 additions).  Afterwards lanes 2i and
-// 2i + 1 both hold the warp sum of value i.  The order of the additions is fixed.
-__device__ __forceinline__ double warp_sum16(double (&v)[16], int lane)
+// 1 / x to FP64 rounding (x normal, > 0): FP32 seed and two Newton steps, 4 FP64 instructions where the
+// division takes about 9.
+__device__ __forceinline__ double recip64(double x)
 {
-#pragma unroll
-    for (int h = 8, off = 16; h >= 1; h >>= 1, off >>= 1) {
-        const bool upper = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const double keep = upper ? v[h + i] : v[i];
-            const double give = upper ? v[i] : v[h + i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
-        }
-    }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+    // seed from the mantissa alone (in [1, 2)), so that no x leaves FP32's range
+    const long long b = __double_as_longlong(x);
+    const double mant = __longlong_as_double((b & 0xfffffffffffffll) | 0x3ff0000000000000ll);
+    const double y0 = f2d_bits(__frcp_rn(d2f_trunc(mant)));
+    const double y1 = fma(y0, fma(-mant, y0, 1.0), y0);
+    const double y2 = fma(y1, fma(-mant, y1, 1.0), y1);  // in (0.5, 1]: exponent 1022 or 1023
+    const int sh = 1023 - (int)((b >> 52) & 0x7ff);
+    return __longlong_as_double(__double_as_longlong(y2) + ((long long)sh << 52));
 }
 
-// Energy terms of particles [p0, p1): per block a fixed-order sum into partial[block][16]; the block
-// that finishes last (ticket from an atomic counter that wraps back to 0) sums the partials in block
-// order into out16.  No thread waits on another block.
+// Energy sums of particles [p0, p1): thread = (particle, DOF), 8 lanes per particle (lanes 0..5 the DOFs,
+// 6 and 7 the accumulators W_int and W_ext), up to kEnergyBlocks blocks striding over the particles, so
+// that a specimen of a few thousand particles fills the chip (one particle per thread, a chain of six
+// divisions each, took 15 us in 15 blocks on 3.7k particles; a step with a read-back there, the two
+// copies of the error words included, went from 65 to 39 us).  Each block writes its
+// 16 sums in a fixed order; the block that finishes last (ticket from an atomic counter that wraps back
+// to 0) adds the partials in block order, and writes them with the handle's non-finite flag and barrier
+// status to out18, which is pinned host memory: the caller waits for the stream and reads them there.
+// No thread waits on another block.
+constexpr int kEnergyBlocks = 304;
 __global__ void __launch_bounds__(256) energy_kernel(DeviceModel m, int32_t p0, int32_t p1, double *partial,
-                                                     unsigned *ticket, double *out16)
+                                                     unsigned *ticket, const int32_t *status, double *out18)
 {
-    __shared__ double red[8][16];
+    __shared__ double red[8][8][3];  // warp, lane class, (kinetic, fixed reaction, prescribed reaction)
     __shared__ bool last;
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int64_t p = (int64_t)p0 + (int64_t)blockIdx.x * 256 + tid;
-    double acc[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc[k] = 0.0;
-    if (p < p1) {
-        const double *ps = m.pstate + 16 * p;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, d = lane & 7;
+    double kin = 0.0, rf = 0.0, rp = 0.0;  // for d = 6, 7 `kin` sums the accumulator
+    for (int64_t p = (int64_t)p0 + (int64_t)blockIdx.x * 32 + (tid >> 3); p < p1; p += 32 * (int64_t)gridDim.x) {
         const double *pd = m.pdyn + 8 * p;
-        const double *pc = m.pconst + 8 * p;
-        const uint64_t bcbits = (uint64_t)__double_as_longlong(pc[6]);
-        const int sp = (int)__double_as_longlong(pc[7]);
-        const SpecDyn &S = m.spec[sp];
-        const double dt = S.dt;
-        const double t = (double)(*m.step) * dt;
-        acc[0] = pd[6];
-        acc[1] = pd[7];
-        for (int d = 0; d < 6; ++d) {
-            const double mass = 1.0 / pc[d];
-            // whole-step velocity v_n from the stored v_{n+1/2} (inverse half kick)
-            const int mk = (int)((bcbits >> (8 * d)) & 0xffu);
-            double v = ps[9 + d];
-            if (mk == 0)
-                v -= S.half_dt * ((m.f_ext ? m.f_ext[6 * p + d] : 0.0) + pd[d]) * pc[d];
-            else if (mk == 1)
-                v = 0.0;
-            else
-                v = m.bc_vel[6 * p + d] * ramp(t, S.inv_ramp);
-            acc[2] += 0.5 * mass * v * v;
-            if (mk == 1) {
-                acc[4 + d] += -pd[d];
-            } else if (mk == 2) {
-                const double ra = ramp(t + 0.5 * dt, S.inv_ramp) - ramp(t - 0.5 * dt, S.inv_ramp);
-                acc[10 + d] += m.bc_vm[6 * p + d] * ra * S.inv_dt - pd[d];
-            }
+        const double fd = pd[d];
+        if (d >= 6) {
+            kin += fd;
+            continue;
         }
+        const double *pc = m.pconst + 8 * p;
+        const double im = pc[d];
+        const int mk = (int)(((uint64_t)__double_as_longlong(pc[6]) >> (8 * d)) & 0xffu);
+        const SpecDyn &S = m.spec[(int)__double_as_longlong(pc[7])];
+        // whole-step velocity v_n from the stored v_{n+1/2} (inverse half kick)
+        double v = 0.0;
+        if (mk == 0) {
+            v = m.pstate[16 * p + 9 + d] - S.half_dt * (m.f_ext ? m.f_ext[6 * p + d] + fd : fd) * im;
+        } else if (mk == 1) {
+            rf -= fd;
+        } else {
+            const double t = (double)(*m.step) * S.dt;
+            v = m.bc_vel[6 * p + d] * ramp(t, S.inv_ramp);
+            const double ra = ramp(t + S.half_dt, S.inv_ramp) - ramp(t - S.half_dt, S.inv_ramp);
+            rp += m.bc_vm[6 * p + d] * ra * S.inv_dt - fd;
+        }
+        if (mk != 1) kin += v * v * recip64(im);
     }
-    const double ws = warp_sum16(acc, lane);
-    if ((lane & 1) == 0) red[w][lane >> 1] = ws;
+#pragma unroll
+    for (int off = 16; off >= 8; off >>= 1) {
+        kin += __shfl_xor_sync(0xffffffffu, kin, off);
+        rf += __shfl_xor_sync(0xffffffffu, rf, off);
+        rp += __shfl_xor_sync(0xffffffffu, rp, off);
+    }
+    if (lane < 8) {
+        red[w][lane][0] = kin;
+        red[w][lane][1] = rf;
+        red[w][lane][2] = rp;
+    }
     __syncthreads();
+    // out: W_int, W_ext, W_kin, pad, fixed reactions (6), prescribed reactions (6)
     if (tid < 16) {
         double b = 0.0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) b += red[k][tid];
+        for (int k = 0; k < 8; ++k) {
+            if (tid < 2) b += red[k][6 + tid][0];
+            if (tid == 2)
+                for (int q = 0; q < 6; ++q) b += 0.5 * red[k][q][0];
+            if (tid >= 4) b += red[k][(tid - 4) % 6][tid < 10 ? 1 : 2];
+        }
         partial[16 * (int64_t)blockIdx.x + tid] = b;
         __threadfence();
     }
     __syncthreads();
     if (tid == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
     __syncthreads();
-    if (last && tid < 16) {
-        double s = 0.0;
-        for (unsigned k = 0; k < gridDim.x; ++k) s += __ldcg(partial + 16 * (int64_t)k + tid);
-        out16[tid] = s;
+    if (!last) return;
+    __shared__ double fin[16][16];
+    const unsigned per = (gridDim.x + 15) / 16;  // partials of one of 16 consecutive runs of blocks
+    double s = 0.0;
+    for (unsigned k = (tid >> 4) * per; k < gridDim.x && k < ((tid >> 4) + 1) * per; ++k)
+        s += __ldcg(partial + 16 * (int64_t)k + (tid & 15));
+    fin[tid >> 4][tid & 15] = s;
+    __syncthreads();
+    if (tid < 16) {
+        double r = 0.0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) r += fin[k][tid];
+        out18[tid] = r;
+    } else if (tid == 16) {
+        out18[16] = (double)*m.flag;
+    } else if (tid == 17) {
+        out18[17] = (double)*status;
     }
 }
 
@@ -1775,11 +1795,11 @@ cudaError_t launch_perturb(const DeviceModel &m, const double *dq, cudaStream_t 
 }
 
 cudaError_t launch_energy(const DeviceModel &m, int32_t p0, int32_t p1, double *partial, unsigned *ticket,
-                          double *out16, cudaStream_t s)
+                          const int32_t *status, double *out18, cudaStream_t s)
 {
-    const int32_t nb = (p1 - p0 + 255) / 256;
-    if (nb <= 0) return cudaMemsetAsync(out16, 0, 16 * sizeof(double), s);
-    energy_kernel<<<nb, 256, 0, s>>>(m, p0, p1, partial, ticket, out16);
+    // an empty range still reports the flags
+    const int nb = std::min(kEnergyBlocks, std::max(1, (p1 - p0 + 31) / 32));
+    energy_kernel<<<nb, 256, 0, s>>>(m, p0, p1, partial, ticket, status, out18);
     return cudaGetLastError();
 }
 
