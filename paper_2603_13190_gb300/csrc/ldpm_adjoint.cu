@@ -321,7 +321,7 @@ __device__ __forceinline__ void facet_law_vjp(const LawConst<R> &c, R l, V3<R> e
     }
 }
 
-// Reverse facet pass of one step (8 tetrahedra, 96 threads per block).
+// Reverse facet pass of one step, mixed mode (8 tetrahedra, 96 threads per block).
 //   phase A  4 threads per tetrahedron: the forward vertex records of the step (as the forward facet
 //            pass), the a_f record, differences to vertex 0; e_V and grad(e_V) per vertex;
 //   phase B  one thread per facet: strain and increment (as forward), a_t = carried - A P^T [[a_f]],
@@ -339,14 +339,14 @@ constexpr int kACon = 24;  // facet contributions: vertex a: q(6) u(6), vertex b
 // 2t, 2t + 1 of each plane (contiguous, no bank conflicts).
 constexpr int kAPlane = 6 * 4 * kATets + 2;
 
-// Mixed mode: 8 resident blocks per SM.  The register cap (80 per thread) costs 24 bytes of spills
-// and doubles the occupancy of the uncapped build; measured 10 % faster on GB300.  The FP64 build
-// (bound by the FP64 pipe) keeps its registers.  S1: one specimen in mixed mode, law constants from
+// 8 resident blocks per SM: the register cap (80 per thread) costs 24 bytes of spills and doubles the
+// occupancy of the uncapped build; measured 10 % faster on GB300.  S1: one specimen, law constants from
 // the kernel parameters (m.law1) instead of the global array, as in the forward facet pass.
-template <class R, bool KT, bool S1>
-__global__ void __launch_bounds__(12 * kATets, sizeof(R) == 4 ? 8 : 1)
+template <bool KT, bool S1>
+__global__ void __launch_bounds__(12 * kATets, 8)
     adjoint_facet_kernel(const __grid_constant__ DeviceModel m, AdjointModel a)
 {
+    using R = float;
     using T4 = R4<R>;
     constexpr int TETS = kATets;
     __shared__ alignas(16) R sv[TETS * 4][kARow + 2];
@@ -385,89 +385,49 @@ __global__ void __launch_bounds__(12 * kATets, sizeof(R) == 4 ? 8 : 1)
         if (tt < m.T) p = reinterpret_cast<const int *>(m.tet)[4 * tt + vi];
         const int base = (threadIdx.x & 31) & ~3;
         R o[kARow], af[kAFr];
-        if constexpr (sizeof(R) == 4) {
-            const float *src = static_cast<const float *>(a.snap_p);
-            float rec[24], arec[12];
-            if (p >= 0) {
-                const float4 *r4 = reinterpret_cast<const float4 *>(src + kMirror * (int64_t)p);
+        const float *src = static_cast<const float *>(a.snap_p);
+        float rec[24], arec[12];
+        if (p >= 0) {
+            const float4 *r4 = reinterpret_cast<const float4 *>(src + kMirror * (int64_t)p);
 #pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    const float4 w = r4[k];
-                    rec[4 * k] = w.x;
-                    rec[4 * k + 1] = w.y;
-                    rec[4 * k + 2] = w.z;
-                    rec[4 * k + 3] = w.w;
-                }
-                const float4 *a4 = reinterpret_cast<const float4 *>(static_cast<const float *>(a.af) + 12 * (int64_t)p);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const float4 w = a4[k];
-                    arec[4 * k] = w.x;
-                    arec[4 * k + 1] = w.y;
-                    arec[4 * k + 2] = w.z;
-                    arec[4 * k + 3] = w.w;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 24; ++k) rec[k] = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 12; ++k) arec[k] = 0.0f;
+            for (int k = 0; k < 6; ++k) {
+                const float4 w = r4[k];
+                rec[4 * k] = w.x;
+                rec[4 * k + 1] = w.y;
+                rec[4 * k + 2] = w.z;
+                rec[4 * k + 3] = w.w;
             }
+            const float4 *a4 = reinterpret_cast<const float4 *>(static_cast<const float *>(a.af) + 12 * (int64_t)p);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const float x0h = __shfl_sync(0xffffffffu, rec[k], base);
-                const float x0l = __shfl_sync(0xffffffffu, rec[3 + k], base);
-                const float u0h = __shfl_sync(0xffffffffu, rec[6 + k], base);
-                const float u0l = __shfl_sync(0xffffffffu, rec[9 + k], base);
-                const float v0 = __shfl_sync(0xffffffffu, rec[15 + k], base);
-                const float a0h = __shfl_sync(0xffffffffu, arec[k], base);
-                const float a0l = __shfl_sync(0xffffffffu, arec[3 + k], base);
-                o[k] = (rec[k] - x0h) + (rec[3 + k] - x0l);
-                o[3 + k] = (rec[6 + k] - u0h) + (rec[9 + k] - u0l);
-                o[6 + k] = rec[15 + k] - v0;
-                o[9 + k] = rec[12 + k];
-                o[12 + k] = rec[18 + k];
-                af[k] = (arec[k] - a0h) + (arec[3 + k] - a0l);
-                af[3 + k] = arec[6 + k];
+                const float4 w = a4[k];
+                arec[4 * k] = w.x;
+                arec[4 * k + 1] = w.y;
+                arec[4 * k + 2] = w.z;
+                arec[4 * k + 3] = w.w;
             }
         } else {
-            const double *src = static_cast<const double *>(a.snap_p);
-            double rec[16], arec[8];
-            if (p >= 0) {
-                const double2 *r2 = reinterpret_cast<const double2 *>(src + 16 * (int64_t)p);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const double2 w = r2[k];
-                    rec[2 * k] = w.x;
-                    rec[2 * k + 1] = w.y;
-                }
-                const double2 *a2 = reinterpret_cast<const double2 *>(static_cast<const double *>(a.af) + 8 * (int64_t)p);
+            for (int k = 0; k < 24; ++k) rec[k] = 0.0f;
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const double2 w = a2[k];
-                    arec[2 * k] = w.x;
-                    arec[2 * k + 1] = w.y;
-                }
-            } else {
+            for (int k = 0; k < 12; ++k) arec[k] = 0.0f;
+        }
 #pragma unroll
-                for (int k = 0; k < 16; ++k) rec[k] = 0.0;
-#pragma unroll
-                for (int k = 0; k < 6; ++k) arec[k] = 0.0;
-            }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const double x0 = __shfl_sync(0xffffffffu, rec[k], base);
-                const double u0 = __shfl_sync(0xffffffffu, rec[3 + k], base);
-                const double v0 = __shfl_sync(0xffffffffu, rec[9 + k], base);
-                const double a0 = __shfl_sync(0xffffffffu, arec[k], base);
-                o[k] = rec[k] - x0;
-                o[3 + k] = rec[3 + k] - u0;
-                o[6 + k] = rec[9 + k] - v0;
-                o[9 + k] = rec[6 + k];
-                o[12 + k] = rec[12 + k];
-                af[k] = arec[k] - a0;
-                af[3 + k] = arec[3 + k];
-            }
+        for (int k = 0; k < 3; ++k) {
+            const float x0h = __shfl_sync(0xffffffffu, rec[k], base);
+            const float x0l = __shfl_sync(0xffffffffu, rec[3 + k], base);
+            const float u0h = __shfl_sync(0xffffffffu, rec[6 + k], base);
+            const float u0l = __shfl_sync(0xffffffffu, rec[9 + k], base);
+            const float v0 = __shfl_sync(0xffffffffu, rec[15 + k], base);
+            const float a0h = __shfl_sync(0xffffffffu, arec[k], base);
+            const float a0l = __shfl_sync(0xffffffffu, arec[3 + k], base);
+            o[k] = (rec[k] - x0h) + (rec[3 + k] - x0l);
+            o[3 + k] = (rec[6 + k] - u0h) + (rec[9 + k] - u0l);
+            o[6 + k] = rec[15 + k] - v0;
+            o[9 + k] = rec[12 + k];
+            o[12 + k] = rec[18 + k];
+            af[k] = (arec[k] - a0h) + (arec[3 + k] - a0l);
+            af[3 + k] = arec[6 + k];
         }
         o[15] = R(0);
         af[6] = af[7] = R(0);
@@ -541,8 +501,8 @@ __global__ void __launch_bounds__(12 * kATets, sizeof(R) == 4 ? 8 : 1)
         const V3<R> ca = {g.x, g.y, g.z};
         const V3<R> cb = ca - d;
         const LawConst<R> *lbase;
-        if constexpr (S1 && sizeof(R) == 4) {
-            lbase = reinterpret_cast<const LawConst<R> *>(&m.law1);
+        if constexpr (S1) {
+            lbase = &m.law1;
         } else {
             const int sp = m.tile_spec ? m.tile_spec[tet0 / 32] : 0;
             lbase = lawc + sp;
@@ -663,6 +623,301 @@ __global__ void __launch_bounds__(12 * kATets, sizeof(R) == 4 ? 8 : 1)
         dst[2 * q + 1] = s[1];
         dst[6 + 2 * q] = s[2];
         dst[6 + 2 * q + 1] = s[3];
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Reverse facet pass of the FP64 mode on edge tiles (5 tetrahedra per warp, one edge with its two facets
+// per lane), as the forward facet_edge_kernel and for the same reason: the FP64 pipe bounds it.  Frames,
+// lengths and grad e_V come from memory; what an edge's facets share is formed once; and a facet that
+// cannot have reached a boundary of the law (FP32 filters of the forward pass) takes the short reverse of
+// the elastic branches, since the adjoints of sigma_bt, sigma_bc and sigma_bs and all that hangs on them
+// are zero there.  The others are collected in shared memory and reversed by full warps with
+// facet_law_vjp.  51k facets: 102 -> 33 us per launch (ncu) against the block kernel.
+// ------------------------------------------------------------------------------------------------
+constexpr int kXRow = 26;     // doubles per staged vertex: forward record (16, 18 with padding), a_f (6)
+constexpr int kXItem = 17;    // doubles per collected facet
+constexpr int kXPlane = 242;  // doubles per contribution plane (20 vertices x 12 values, padded)
+constexpr int kXWords = 12 * kEdgeTets * kXItem;  // per warp; rows (520) and planes (726) lie in them
+static_assert(4 * kEdgeTets * kXRow <= kXWords && 3 * kXPlane <= kXWords, "rows and planes fit");
+constexpr int kXWarps = 2;
+
+template <bool KT>
+__global__ void __launch_bounds__(32 * kXWarps)
+    adjoint_edge_kernel(const __grid_constant__ DeviceModel m, AdjointModel a)
+{
+    __shared__ alignas(16) double sw_[kXWarps][kXWords];
+    const int lane = threadIdx.x & 31;
+    double *sw = sw_[threadIdx.x >> 5];
+    const int64_t tet0l = ((int64_t)blockIdx.x * kXWarps + (threadIdx.x >> 5)) * kEdgeTets;
+    if (tet0l >= m.T) return;  // the whole warp
+    const int32_t tet0 = (int32_t)tet0l;
+    const int j = lane / 6, e = lane - 6 * j, jj = j < kEdgeTets ? j : 0;
+    const int32_t tt = tet0 + j;
+    const bool in = lane < 6 * kEdgeTets && tt < m.T;
+    // ---- records to shared memory: pieces 1..7 of the forward record, 3 of a_f
+    int vid = -1;
+    if (lane < 4 * kEdgeTets && tet0 + (lane >> 2) < m.T)
+        vid = __ldg(reinterpret_cast<const int *>(m.tet) + 4 * (int64_t)tet0 + lane);
+    const double *rec = static_cast<const double *>(a.snap_p), *afr = static_cast<const double *>(a.af);
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const int c = lane + 32 * i;
+        const int v = c / 10, part = c - 10 * v;
+        const int id = __shfl_sync(0xffffffffu, vid, v & 31);
+        if (c < 40 * kEdgeTets) {
+            const int64_t p = id >= 0 ? id : 0;
+            const double *src = part < 7 ? rec + 16 * p + 2 * (part + 1) : afr + 8 * p + 2 * (part - 7);
+            cp_async16<false>(sw + kXRow * v + (part < 7 ? 2 * (part + 1) : 18 + 2 * (part - 7)), src, id >= 0);
+        }
+    }
+    const bool live = __shfl_sync(0xffffffffu, vid, 4 * jj) >= 0 && in;
+    const int64_t f = 12 * (int64_t)tt + 2 * e;
+    V3<double> P0{}, P1{}, P2{}, d{}, gr{};
+    double lA[2] = {}, l = 1.0, ht = 0.0;
+    if (live) {
+        const double2 *fr = reinterpret_cast<const double2 *>(m.frame) + 8 * (6 * (int64_t)tt + e);
+        const double2 a0 = __ldg(fr), a1 = __ldg(fr + 1), a2 = __ldg(fr + 2), a3 = __ldg(fr + 3), a4 = __ldg(fr + 4),
+                      a5 = __ldg(fr + 5), a6 = __ldg(fr + 6), a7 = __ldg(fr + 7);
+        P0 = {a0.x, a0.y, a1.x};
+        P1 = {a1.y, a2.x, a2.y};
+        P2 = {a3.x, a3.y, a4.x};
+        d = {a4.y, a5.x, a5.y};
+        lA[0] = a6.x;
+        lA[1] = a6.y;
+        l = a7.x;
+        ht = a7.y;
+        if (e < 3) {
+            const double *g3 = m.grad + 3 * (3 * (int64_t)tt + e);
+            gr = {__ldg(g3), __ldg(g3 + 1), __ldg(g3 + 2)};
+        }
+    }
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    const int va = (0x211000 >> (4 * e)) & 0xF, vb = (0x332321 >> (4 * e)) & 0xF;
+    V3<double> wq, wv, wf, dth, dom, dta;
+    double eV;
+    {
+        // record: x 0..2, u 3..5, theta 6..8, v 9..11, omega 12..14; a_f 18..23
+        const double *A = sw + kXRow * (4 * jj + va), *B = sw + kXRow * (4 * jj + vb);
+        const V3<double> du = {B[3] - A[3], B[4] - A[4], B[5] - A[5]};
+        const V3<double> thB = {B[6], B[7], B[8]}, omB = {B[12], B[13], B[14]}, taB = {B[21], B[22], B[23]};
+        dth = {thB.x - A[6], thB.y - A[7], thB.z - A[8]};
+        dom = {omB.x - A[12], omB.y - A[13], omB.z - A[14]};
+        dta = {taB.x - A[21], taB.y - A[22], taB.z - A[23]};
+        wq = add_cross(du, d, thB);
+        wv = add_cross(V3<double>{B[9] - A[9], B[10] - A[10], B[11] - A[11]}, d, omB);
+        wf = add_cross(V3<double>{B[18] - A[18], B[19] - A[19], B[20] - A[20]}, d, taB);
+        const double term = fma(gr.x, du.x, fma(gr.y, du.y, gr.z * du.z));
+        const int base = 6 * jj;
+        eV = __shfl_sync(0xffffffffu, term, base) + __shfl_sync(0xffffffffu, term, base + 1) +
+             __shfl_sync(0xffffffffu, term, base + 2);
+    }
+    __syncwarp();  // the rows are read
+    const LawConst<double> &c = *static_cast<const LawConst<double> *>(m.law);
+    const double dt = c.dt;
+    const double4a *__restrict__ geo = static_cast<const double4a *>(m.geo);
+    double4a *__restrict__ adj_h = static_cast<double4a *>(a.adj_h);
+    double4a *__restrict__ gacc = static_cast<double4a *>(a.gacc);
+    auto proj = [&](V3<double> J) -> V3<double> {
+        return {fma(P0.x, J.x, fma(P0.y, J.y, P0.z * J.z)), fma(P1.x, J.x, fma(P1.y, J.y, P1.z * J.z)),
+                fma(P2.x, J.x, fma(P2.y, J.y, P2.z * J.z))};
+    };
+    auto lift = [&](V3<double> t) -> V3<double> {
+        return {fma(t.x, P0.x, fma(t.y, P1.x, t.z * P2.x)), fma(t.x, P0.y, fma(t.y, P1.y, t.z * P2.y)),
+                fma(t.x, P0.z, fma(t.y, P1.z, t.z * P2.z))};
+    };
+    V3<double> SG{}, MG{}, SD{}, MD{};  // sums over the two facets: displacement and velocity adjoints
+    double aeV = 0.0;
+    auto finish = [&](int i, V3<double> arm, const LawVJP<double> &o) {
+        double4a nc;
+        nc.x = o.atN;
+        nc.y = o.atM;
+        nc.z = o.atL;
+        nc.w = o.aemax;
+        adj_h[f + i] = nc;
+        double4a ga = gacc[f + i];
+        ga.x += o.gE0;
+        ga.y += o.galpha;
+        ga.z += o.gsigma;
+        gacc[f + i] = ga;
+        aeV += o.aeV;
+        const V3<double> Ge = lift(o.ae), Gd = dt * lift(o.ade);
+        SG = SG + Ge;
+        MG = add_cross(MG, arm, Ge);
+        SD = SD + Gd;
+        MD = add_cross(MD, arm, Gd);
+    };
+    bool need[2] = {false, false};
+    int items = 0, slot[2] = {0, 0};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        V3<double> es{}, de{}, at{}, arm{};
+        double4a h{};
+        double ah = 0.0;
+        if (live) {
+            const double4a g = geo[f + i], car = adj_h[f + i];
+            h = static_cast<const double4a *>(a.snap_h)[f + i];
+            arm = {g.x, g.y, g.z};
+            es = proj(add_cross(wq, dth, arm));
+            de = dt * proj(add_cross(wv, dom, arm));
+            const V3<double> jf = proj(add_cross(wf, dta, arm));
+            at = {fma(-lA[i], jf.x, car.x), fma(-lA[i], jf.y, car.y), fma(-lA[i], jf.z, car.z)};
+            ah = car.w;
+            FacetPar64 fp = {c.E0, c.alpha, c.inv_alpha, c.sigma_t};
+            if (m.pf) {
+                const double4a pp = static_cast<const double4a *>(m.pf)[f + i];
+                fp = {pp.x, pp.y, pp.w, pp.z};
+            }
+            LawVJP<double> o;
+            o.aeV = o.gsigma = 0.0;
+            o.aemax = ah;
+            const double aE = fp.alpha * fp.E0;
+            if (c.elastic) {  // t = E0 (e_N, alpha e_M, alpha e_L)
+                const double sT = es.y * at.y + es.z * at.z;
+                o.ae = {fp.E0 * at.x, aE * at.y, aE * at.z};
+                o.ade = {0.0, 0.0, 0.0};
+                o.atN = o.atM = o.atL = 0.0;
+                o.gE0 = es.x * at.x + fp.alpha * sT;
+                o.galpha = fp.E0 * sT;
+            } else if (order_bits(es.x) <= 0) {
+                V3<double> tr = {h.x, h.y, h.z};
+                need[i] = compression_trial64(c, fp, de, tr);
+                const bool below = order_bits(-h.x) <= order_bits(c.sigma_c0);
+                const double ENc = below ? fp.E0 : c.Ed_E0 * fp.E0;
+                const double a_tns = order_bits(h.x + ENc * de.x) > 0 ? 0.0 : at.x;
+                const double sdd = de.y * at.y + de.z * at.z;
+                o.ae = {0.0, 0.0, 0.0};
+                o.ade = {ENc * a_tns, aE * at.y, aE * at.z};
+                o.atN = a_tns;
+                o.atM = at.y;
+                o.atL = at.z;
+                o.gE0 = fp.alpha * sdd + (below ? de.x : c.Ed_E0 * de.x) * a_tns;
+                o.galpha = fp.E0 * sdd;
+            } else {
+                const double eT2 = es.y * es.y + es.z * es.z, a2 = fp.alpha * eT2;
+                const double e2 = es.x * es.x + a2;
+                const V3<double> ep = es - de;
+                const double epT2 = ep.y * ep.y + ep.z * ep.z;
+                const double eo2 = ep.x * ep.x + fp.alpha * epT2;
+                const double tT2 = h.y * h.y + h.z * h.z;
+                const double to2 = h.x * h.x + tT2 * fp.inv_alpha;
+                const double ie = rsqrt(e2), eff = e2 * ie;
+                // sqrt'(0) = 0
+                const double ieo = order_bits(eo2) > 0 ? rsqrt(eo2) : 0.0, ito = order_bits(to2) > 0 ? rsqrt(to2) : 0.0;
+                const double num = de.x * (es.x + ep.x) + fp.alpha * (de.y * (es.y + ep.y) + de.z * (es.z + ep.z));
+                const double d_eff = num / (eff + eo2 * ieo);
+                const double ts = to2 * ito + fp.E0 * d_eff;
+                const double t1 = order_bits(ts) < 0 ? 0.0 : ts;
+                const bool keep = order_bits(h.w) > order_bits(eff);
+                const double em = keep ? h.w : eff;
+                need[i] = order_bits(e2) < order_bits(1e-300) || (KT && c.k_t > 0.0 && order_bits(to2) <= 0) ||
+                          !fracture_inside32(c, fp, t1, es.x, a2, ie, em, ht);
+                // the trial stands: out = r (e_N, alpha e_M, alpha e_L), r = t / e, t = <t_old + E0 d_eff>
+                const double r = t1 * ie;
+                const double sT = es.y * at.y + es.z * at.z;
+                const double a_r = es.x * at.x + fp.alpha * sT, ar = fp.alpha * r;
+                const double a_ts = order_bits(ts) < 0 ? 0.0 : a_r * ie;
+                const double a_de = fp.E0 * a_ts;
+                const double ko = -a_de * ieo, kt = a_ts * ito;
+                double a_eff = a_de - r * ie * a_r;
+                if (!keep) {
+                    a_eff += ah;
+                    o.aemax = 0.0;
+                }
+                const double ke = a_eff * ie, kea = fp.alpha * ke, koa = fp.alpha * ko;
+                const V3<double> a_ep = {ko * ep.x, koa * ep.y, koa * ep.z};
+                o.ae = {r * at.x + ke * es.x + a_ep.x, ar * at.y + kea * es.y + a_ep.y, ar * at.z + kea * es.z + a_ep.z};
+                o.ade = {-a_ep.x, -a_ep.y, -a_ep.z};
+                o.atN = kt * h.x;
+                o.atM = kt * fp.inv_alpha * h.y;
+                o.atL = kt * fp.inv_alpha * h.z;
+                o.gE0 = d_eff * a_ts;
+                o.galpha = r * sT + 0.5 * (ko * epT2 + ke * eT2 - kt * tT2 * fp.inv_alpha * fp.inv_alpha);
+            }
+            if (!need[i]) finish(i, arm, o);
+        }
+        // collect the others
+        const unsigned b = __ballot_sync(0xffffffffu, need[i]);
+        slot[i] = items + __popc(b & ((1u << lane) - 1u));
+        items += __popc(b);
+        if (need[i]) {
+            double *w = sw + kXItem * slot[i];
+            const double v[kXItem] = {l, es.x, es.y, es.z, de.x, de.y, de.z, eV, h.x, h.y, h.z, h.w, at.x, at.y, at.z,
+                                      ah, __longlong_as_double(f + i)};
+#pragma unroll
+            for (int k = 0; k < kXItem; ++k) w[k] = v[k];
+        }
+    }
+    if (items) {
+        __syncwarp();
+        for (int k = lane; k < items; k += 32) {
+            double *w = sw + kXItem * k;
+            LawConst<double> cp = c;
+            if (m.pf) {
+                const double4a pp = static_cast<const double4a *>(m.pf)[__double_as_longlong(w[16])];
+                cp = facet_params(c, pp.x, pp.y, pp.z);
+            }
+            LawVJP<double> o;
+            facet_law_vjp<double, KT>(cp, w[0], V3<double>{w[1], w[2], w[3]}, V3<double>{w[4], w[5], w[6]}, w[7], w[8],
+                                      w[9], w[10], w[11], w[12], w[13], w[14], w[15], o);
+            const double v[14] = {o.ae.x, o.ae.y, o.ae.z, o.ade.x, o.ade.y, o.ade.z, o.aeV, o.atN, o.atM, o.atL,
+                                  o.aemax, o.gE0, o.galpha, o.gsigma};
+#pragma unroll
+            for (int q = 0; q < 14; ++q) w[q] = v[q];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (need[i]) {
+                const double *w = sw + kXItem * slot[i];
+                const LawVJP<double> o = {{w[0], w[1], w[2]}, {w[3], w[4], w[5]}, w[6],  w[7], w[8],
+                                          w[9],               w[10],              w[11], w[12], w[13]};
+                const double4a g = geo[f + i];
+                finish(i, V3<double>{g.x, g.y, g.z}, o);
+            }
+        __syncwarp();
+    }
+    // vertex a receives (-S, -M) of either adjoint, vertex b (S, M - d x S); vertices 1..3 also receive
+    // grad(e_V) times the tetrahedron's summed a_eV, vertex 0 minus their sum
+    V3<double> ga{}, gb{};
+    if (__any_sync(0xffffffffu, __double_as_longlong(aeV) != 0)) {
+        double aT = 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) aT += __shfl_sync(0xffffffffu, aeV, 6 * jj + k);
+        gb = aT * gr;  // gr is zero on the edges 3..5
+    }
+    ga = V3<double>{-SG.x, -SG.y, -SG.z} - gb;
+    gb = SG + gb;
+    const unsigned lv = __ballot_sync(0xffffffffu, live);
+    if (live) {
+        const int ka = (0x221210 >> (4 * e)) & 0xF, kb = (0x211000 >> (4 * e)) & 0xF;
+        const V3<double> Mq = add_cross(MG, SG, d), Mu = add_cross(MD, SD, d);
+        double2 *da = reinterpret_cast<double2 *>(sw + ka * kXPlane + 12 * (4 * j + va));
+        double2 *db = reinterpret_cast<double2 *>(sw + kb * kXPlane + 12 * (4 * j + vb));
+        da[0] = double2{ga.x, ga.y};
+        da[1] = double2{ga.z, -MG.x};
+        da[2] = double2{-MG.y, -MG.z};
+        da[3] = double2{-SD.x, -SD.y};
+        da[4] = double2{-SD.z, -MD.x};
+        da[5] = double2{-MD.y, -MD.z};
+        db[0] = double2{gb.x, gb.y};
+        db[1] = double2{gb.z, Mq.x};
+        db[2] = double2{Mq.y, Mq.z};
+        db[3] = double2{SD.x, SD.y};
+        db[4] = double2{SD.z, Mu.x};
+        db[5] = double2{Mu.y, Mu.z};
+    }
+    __syncwarp();
+    double2 *__restrict__ out = reinterpret_cast<double2 *>(static_cast<double *>(a.tvc2) + 48 * (int64_t)tet0);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int q = lane + 30 * i;  // pair q of the tile's 240 values
+        if (lane < 30 && ((lv >> (6 * (q / 24))) & 1u)) {
+            const double2 *s2 = reinterpret_cast<const double2 *>(sw) + q;
+            const double2 x = s2[0], y = s2[kXPlane / 2], z = s2[kXPlane];
+            out[q] = double2{(x.x + y.x) + z.x, (x.y + y.y) + z.y};
+        }
     }
 }
 
@@ -868,19 +1123,27 @@ cudaError_t launch_adjoint_init(const DeviceModel &m, const AdjointModel &a, cud
 template <class R>
 cudaError_t launch_adjoint_facet(const DeviceModel &m, const AdjointModel &a, cudaStream_t s)
 {
-    const unsigned fblocks = (unsigned)((m.T + kATets - 1) / kATets);
-    if (fblocks) {
-        const bool s1 = sizeof(R) == 4 && m.n_spec == 1;
+    if (m.T <= 0) return cudaSuccess;
+    if constexpr (sizeof(R) == 8) {
+        const int64_t tiles = ((int64_t)m.T + kEdgeTets - 1) / kEdgeTets;
+        const unsigned nb = (unsigned)((tiles + kXWarps - 1) / kXWarps);
+        if (a.reload)
+            adjoint_edge_kernel<true><<<nb, 32 * kXWarps, 0, s>>>(m, a);
+        else
+            adjoint_edge_kernel<false><<<nb, 32 * kXWarps, 0, s>>>(m, a);
+    } else {
+        const unsigned nb = (unsigned)((m.T + kATets - 1) / kATets);
+        const bool s1 = m.n_spec == 1;
         if (a.reload) {
             if (s1)
-                adjoint_facet_kernel<R, true, true><<<fblocks, 12 * kATets, 0, s>>>(m, a);
+                adjoint_facet_kernel<true, true><<<nb, 12 * kATets, 0, s>>>(m, a);
             else
-                adjoint_facet_kernel<R, true, false><<<fblocks, 12 * kATets, 0, s>>>(m, a);
+                adjoint_facet_kernel<true, false><<<nb, 12 * kATets, 0, s>>>(m, a);
         } else {
             if (s1)
-                adjoint_facet_kernel<R, false, true><<<fblocks, 12 * kATets, 0, s>>>(m, a);
+                adjoint_facet_kernel<false, true><<<nb, 12 * kATets, 0, s>>>(m, a);
             else
-                adjoint_facet_kernel<R, false, false><<<fblocks, 12 * kATets, 0, s>>>(m, a);
+                adjoint_facet_kernel<false, false><<<nb, 12 * kATets, 0, s>>>(m, a);
         }
     }
     return cudaGetLastError();

@@ -248,6 +248,19 @@ __device__ __forceinline__ float fracture_floor32(float E0, float four_a_r2, flo
     return 0.9999f * s0 * exp_(-1.0001f * H0 * over / s0);
 }
 
+// Whether the trial effective traction t surely stays below the fracture boundary.
+__device__ __forceinline__ bool fracture_inside32(const LawConst<double> &c, const FacetPar64 &f, double t, double eN,
+                                                  double aT2, double inv_e, double emax, double ht)
+{
+    const float E0 = d2f_trunc(f.E0), st = d2f_trunc(f.sigma_t), tf = d2f_trunc(t), em = d2f_trunc(emax);
+    const float al = d2f_trunc(f.alpha), k4 = al * d2f_trunc(c.four_over_r2);
+    // sigma_0 >= 2 sigma_t / (1 + sqrt(max(1, 4 alpha / r_st^2))) for every omega
+    const float s0min = 0.9999f * 2.0f * st / (1.0f + sqrtf(fmaxf(1.0f, k4)));
+    if (E0 * em <= s0min && tf <= s0min) return true;
+    return tf <= 0.9999f * fracture_floor32(E0, k4, d2f_trunc(c.r_s) * E0 / al, st, d2f_trunc(c.n_t), d2f_trunc(eN),
+                                            d2f_trunc(aT2), d2f_trunc(inv_e), em, d2f_trunc(ht));
+}
+
 // Compression and friction (App. A.2, A.3) of one facet, eN <= 0.  The trial: t in, the elastic trial
 // out, with t_N <= 0 applied where that is all.  Returns whether a boundary may be reached, in which
 // case compression_return64 has to follow.
@@ -301,6 +314,20 @@ __device__ __forceinline__ void compression_return64(const LawConst<double> &c, 
         t.z *= s;
     }
     t.x = tn;
+}
+
+constexpr int kEdgeTets = 5;  // tetrahedra per warp of the FP64 edge tiles (30 of 32 lanes own an edge)
+
+// 16-byte asynchronous copy into shared memory; zeros with `ok` false.  PERSIST: through L2 only.
+template <bool PERSIST>
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = ok ? 16 : 0;
+    if constexpr (PERSIST)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
 }
 
 template <class R>

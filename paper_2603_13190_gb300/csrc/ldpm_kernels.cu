@@ -556,25 +556,12 @@ __global__ void __launch_bounds__(32 * WPB, 12)
 // launch on GB300 (ncu): 594 -> 225 us on 676k facets in tension past the peak, 540 -> 270 us on 1.15M
 // facets in compression; the FP64 pipe is 86 % busy in both.
 // ------------------------------------------------------------------------------------------------
-constexpr int kEdgeTets = 5;
 constexpr int kERow = 18;       // doubles per staged vertex record (16, padded against bank conflicts)
 constexpr int kEPlane = 122;    // doubles per contribution plane (20 vertices x 6 values, padded)
 constexpr int kEItem = 7;       // doubles per collected facet
 constexpr int kEWords = 12 * kEdgeTets * kEItem;  // doubles per warp; rows (360) and planes (366) lie in them
 static_assert(4 * kEdgeTets * kERow <= kEWords && 3 * kEPlane <= kEWords, "rows and planes fit");
 constexpr int kEdgeWarps = 2;   // warps (tiles) per block
-
-// 16-byte asynchronous copy into shared memory; zeros with `ok` false.  PERSIST: through L2 only.
-template <bool PERSIST>
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    const int n = ok ? 16 : 0;
-    if constexpr (PERSIST)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-}
 
 // Tetrahedra [tet0, tet0 + 5) by one warp on its own shared words sw (a tile may straddle two specimens:
 // the law constants are read per lane).
@@ -709,14 +696,7 @@ __device__ __forceinline__ void facet_edge_tile(const DeviceModel &m, const doub
             }
             double tr = fma(fp.E0, d_eff, t_old);
             tr = order_bits(tr) < 0 ? 0.0 : tr;
-            const float E0f = d2f_trunc(fp.E0), stf = d2f_trunc(fp.sigma_t), trf = d2f_trunc(tr), emf = d2f_trunc(em);
-            const float k4 = d2f_trunc(fp.alpha) * d2f_trunc(c.four_over_r2);
-            // sigma_0 >= 2 sigma_t / (1 + sqrt(max(1, 4 alpha / r_st^2))) for every omega
-            const float s0min = 0.9999f * 2.0f * stf / (1.0f + sqrtf(fmaxf(1.0f, k4)));
-            need[i] = !(E0f * emf <= s0min && trf <= s0min) &&
-                      !(trf <= fracture_floor32(E0f, k4, d2f_trunc(c.r_s) * E0f / d2f_trunc(fp.alpha), stf,
-                                                d2f_trunc(c.n_t), d2f_trunc(es.x), d2f_trunc(a2), d2f_trunc(ie), emf,
-                                                d2f_trunc(ht)) * 0.9999f);
+            need[i] = !fracture_inside32(c, fp, tr, es.x, a2, ie, em, ht);
             t[i].x = tr;
             emax[i] = em;
             inv_e[i] = ie;
