@@ -217,6 +217,8 @@ struct ldpm_ctx {
     std::vector<int64_t> ufoff;         // [n_spec + 1] offsets of each specimen's facets in d_umap
     double *d_scratch = nullptr;        // state read-back scratch, grown on demand
     size_t scratch_n = 0;
+    char *d_adj = nullptr;              // workspace of ldpm_adjoint, kept between calls up to kAdjointKeep bytes
+    size_t adj_bytes = 0;
     std::map<int64_t, cudaGraphExec_t> graphs;
     bool prof = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -243,7 +245,7 @@ void free_model(ldpm_ctx *h)
                     h->dm.geo,
                     h->dm.hist, h->dm.fout, h->dm.tvc, h->dm.ent, h->dm.row, h->dm.stab, h->dm.tile_spec, h->dm.law, h->dm.spec,
                     h->dm.step, h->dm.flag, h->d_partial, h->dm.pf, h->d_umap, h->d_scratch, h->d_ticket,
-                    h->d_pmap, h->pctl.arrive, h->pctl.status, h->dm.frame, h->dm.grad};
+                    h->d_pmap, h->pctl.arrive, h->pctl.status, h->dm.frame, h->dm.grad, h->d_adj};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->h_out18) cudaFreeHost(h->h_out18);
@@ -1340,6 +1342,8 @@ size_t slot_stride(const ldpm_ctx *h)
     return align256(b.ps) + align256(b.pd) + align256(b.pm) + align256(b.hist) + 256;
 }
 
+constexpr size_t kAdjointKeep = (size_t)512 << 20;
+
 template <class R>
 int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J, double *gE0, double *galpha,
                 double *gsigma)
@@ -1362,24 +1366,55 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
     const size_t rec = mixed ? (size_t)kMirror * N * sizeof(float) : 16 * (size_t)N * sizeof(double);
     const size_t hb = (size_t)Fint * sizeof(R4<R>);
     const size_t snap_stride = align256(rec) + align256(hb);
+    // One workspace: allocating and freeing a dozen buffers costs a small model as much as its reverse
+    // pass, so it stays with the handle (until ldpm_destroy) while it is no larger than kAdjointKeep; a larger
+    // one lives for the call.  The output buffer (3 F doubles) lies over adj_h and gacc, whose contents the
+    // totals no longer need when it is written.
     DevArena ar;
     char *ckpt = nullptr, *snap = nullptr;
     AdjointModel a;
     for (auto &sp : h->sp) a.reload |= sp.mat.k_t > 0.0;
-    if ((rc = ar.get(&ckpt, stride * (size_t)(nseg + 1))) || (rc = ar.get(&snap, snap_stride * (size_t)std::min(C, K))))
-        return fail(LDPM_E_OOM, "adjoint: %lld checkpoints of %zu bytes and %lld step snapshots of %zu bytes do "
-                                "not fit (use a smaller checkpoint interval)",
-                    (long long)(nseg + 1), stride, (long long)std::min(C, K), snap_stride);
-    if ((rc = ar.get((double **)&a.cseed, 6 * (size_t)N)) || (rc = ar.get(&a.Qbar, 6 * (size_t)N)) ||
-        (rc = ar.get(&a.Ubar, 6 * (size_t)N)) || (rc = ar.get(&a.jacc, (size_t)N)) ||
-        (rc = ar.get((R4<R> **)&a.adj_h, (size_t)Fint)) || (rc = ar.get((R4<R> **)&a.gacc, (size_t)Fint)) ||
-        (rc = ar.get((R **)&a.tvc2, 4 * (size_t)Fint)))
-        return rc;
-    if (mixed) {
-        if ((rc = ar.get((float **)&a.af, 12 * (size_t)N)) || (rc = ar.get(&a.gsum, 4 * (size_t)Fint))) return rc;
+    const size_t n6 = 6 * (size_t)N * sizeof(double), af = (size_t)N * (mixed ? 12 * sizeof(float) : 8 * sizeof(double));
+    size_t off = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = off;
+        off += align256(bytes);
+        return at;
+    };
+    const size_t o_ckpt = part(stride * (size_t)(nseg + 1)), o_snap = part(snap_stride * (size_t)std::min(C, K)),
+                 o_c = part(n6), o_Q = part(n6), o_U = part(n6), o_j = part((size_t)N * sizeof(double)), o_af = part(af),
+                 o_h = part(hb), o_g = part(hb), o_t = part(4 * (size_t)Fint * sizeof(R)),
+                 o_s = part(mixed ? 4 * (size_t)Fint * sizeof(double) : 0), o_bad = part(sizeof(int32_t));
+    char *ws = nullptr;
+    if (off <= kAdjointKeep && h->adj_bytes >= off) {
+        ws = h->d_adj;
     } else {
-        if ((rc = ar.get((double **)&a.af, 8 * (size_t)N))) return rc;
+        if (h->d_adj) cudaFree(h->d_adj);  // the stream is idle (ldpm_adjoint has waited for it)
+        h->d_adj = nullptr;
+        h->adj_bytes = 0;
+        if ((rc = dalloc(&ws, off)))
+            return fail(LDPM_E_OOM, "adjoint: %lld checkpoints of %zu bytes and %lld step snapshots of %zu bytes do "
+                                    "not fit (use a smaller checkpoint interval)",
+                        (long long)(nseg + 1), stride, (long long)std::min(C, K), snap_stride);
+        if (off <= kAdjointKeep) {
+            h->d_adj = ws;
+            h->adj_bytes = off;
+        } else {
+            ar.ptrs.push_back(ws);
+        }
     }
+    ckpt = ws + o_ckpt;
+    snap = ws + o_snap;
+    a.cseed = (double *)(ws + o_c);
+    a.Qbar = (double *)(ws + o_Q);
+    a.Ubar = (double *)(ws + o_U);
+    a.jacc = (double *)(ws + o_j);
+    a.af = ws + o_af;
+    a.adj_h = ws + o_h;
+    a.gacc = ws + o_g;
+    a.tvc2 = ws + o_t;
+    if (mixed) a.gsum = (double *)(ws + o_s);
+    int32_t *d_bad = (int32_t *)(ws + o_bad);
     CU(cudaMemcpyAsync(a.cseed, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     CU(cudaMemsetAsync(a.jacc, 0, (size_t)N * sizeof(double), h->stream));
     auto fwd = [&](bool objective) -> int {
@@ -1459,24 +1494,28 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
     // results
     std::vector<double> jp((size_t)N);
     CU(cudaMemcpyAsync(jp.data(), a.jacc, jp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    std::vector<double> g4(grads ? 4 * (size_t)Fint : 0);
-    if (grads)
-        CU(cudaMemcpyAsync(g4.data(), mixed ? (const void *)a.gsum : (const void *)a.gacc, g4.size() * sizeof(double),
-                           cudaMemcpyDeviceToHost, h->stream));
+    int32_t bad = 0;
+    double *outs[3] = {gE0, galpha, gsigma};
+    if (grads) {
+        // to the caller's facet order on the device, then straight into the caller's arrays
+        double *d3 = (double *)a.adj_h;
+        const double *src = mixed ? a.gsum : (const double *)a.gacc;
+        CU(cudaMemsetAsync(d_bad, 0, sizeof(int32_t), h->stream));
+        CU(launch_grad_to_user(src, h->d_umap, S.F, d3, d_bad, h->stream));
+        for (int k3 = 0; k3 < 3; ++k3)
+            if (outs[k3])
+                CU(cudaMemcpyAsync(outs[k3], d3 + (size_t)k3 * S.F, (size_t)S.F * sizeof(double), cudaMemcpyDeviceToHost,
+                                   h->stream));
+        CU(cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, h->stream));
+    }
     CU(cudaStreamSynchronize(h->stream));
     if (J) {
         double acc = 0.0;
         for (double x : jp) acc += x;
         *J = acc;
     }
-    double *outs[3] = {gE0, galpha, gsigma};
     for (int k3 = 0; k3 < 3; ++k3)
-        if (outs[k3])
-            for (int32_t k = 0; k < S.F; ++k) outs[k3][k] = g4[4 * (size_t)S.fmap[k] + k3];
-    for (int k3 = 0; k3 < 3; ++k3)
-        if (outs[k3])
-            for (int32_t k = 0; k < S.F; ++k)
-                if (!std::isfinite(outs[k3][k])) return fail(LDPM_E_UNSTABLE, "adjoint: non-finite gradient");
+        if (outs[k3] && ((bad >> k3) & 1)) return fail(LDPM_E_UNSTABLE, "adjoint: non-finite gradient");
     return LDPM_OK;
 }
 

@@ -209,6 +209,10 @@ cudaError_t launch_adjoint_gather(const DeviceModel &m, const AdjointModel &a, c
 // gsum += gacc, gacc = 0 (mixed mode, at the end of each reversed segment).
 template <class R>
 cudaError_t launch_adjoint_fold(const DeviceModel &m, const AdjointModel &a, cudaStream_t s);
+// Gradients of n facets in the caller's order: out3[c n + k] = src[4 f + c], f = umap[k] / 2, c = 0..2; bit c
+// of *bad (0 before) is set if a value of component c is not finite.
+cudaError_t launch_grad_to_user(const double *src, const int32_t *umap, int64_t n, double *out3, int32_t *bad,
+                                cudaStream_t s);
 // After a forward step (node forces f_n in pdyn, step counter n): jacc[p] += sum_d seed_pd R_pd(t_n) / K
 // with seed / K = -c, i.e. the particle's share of the objective.
 cudaError_t launch_objective(const DeviceModel &m, const AdjointModel &a, cudaStream_t s);
