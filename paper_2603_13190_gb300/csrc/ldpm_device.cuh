@@ -170,18 +170,22 @@ __device__ __forceinline__ void facet_law(const LawConst<R> &c, R l, V3<R> e, V3
     R tn = tN + ENc * de.x;
     const R eD = e.x - eV;
     const R eDV = eV + c.beta * eD;
-    const R rDV = (eV <= R(0)) ? -fabs(eD) / (eV - c.eV0) : fabs(eD) / c.eV0;
-    const R mac = rDV - c.kc1 > R(0) ? rDV - c.kc1 : R(0);
-    const R Hc = (c.Hc0 - c.Hc1) / (R(1) + c.kc2 * mac) + c.Hc1;
-    R sigma_bc;
-    if (-eDV <= R(0)) {
-        sigma_bc = c.sigma_c0;
-    } else if (-eDV <= c.ec1) {
-        const R o = -eDV - c.ec0 > R(0) ? -eDV - c.ec0 : R(0);
-        sigma_bc = c.sigma_c0 + o * Hc;
-    } else {
-        const R sigma_c1 = c.sigma_c0 + (c.ec1 - c.ec0) * Hc;
-        sigma_bc = sigma_c1 * exp_((-eDV - c.ec1) * Hc / sigma_c1);
+    // the hardening modulus H_c matters only past the elastic compaction e_c0: below it the boundary is
+    // sigma_c0 (the two divisions of H_c skipped: 4 % of the mixed step on 11.4M facets in compression).
+    // Guarding the fracture boundary in the same way was slower past the peak, where nearly every warp
+    // has a facet that needs it: 2.0M facets 1019 -> 1043 us per 20 steps.
+    R sigma_bc = c.sigma_c0;
+    if (-eDV > c.ec0) {
+        const R rDV = (eV <= R(0)) ? -fabs(eD) / (eV - c.eV0) : fabs(eD) / c.eV0;
+        const R mac = rDV - c.kc1 > R(0) ? rDV - c.kc1 : R(0);
+        const R Hc = (c.Hc0 - c.Hc1) / (R(1) + c.kc2 * mac) + c.Hc1;
+        if (-eDV <= c.ec1) {
+            const R o = -eDV - c.ec0;
+            sigma_bc = c.sigma_c0 + o * Hc;
+        } else {
+            const R sigma_c1 = c.sigma_c0 + (c.ec1 - c.ec0) * Hc;
+            sigma_bc = sigma_c1 * exp_((-eDV - c.ec1) * Hc / sigma_c1);
+        }
     }
     tn = tn < -sigma_bc ? -sigma_bc : tn;
     tn = tn > R(0) ? R(0) : tn;

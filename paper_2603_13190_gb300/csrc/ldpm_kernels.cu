@@ -194,10 +194,10 @@ __device__ __forceinline__ void stage_vertex(const DeviceModel &m, const void *_
 // and its contributions to its two vertices in cs[12] (zeros when the facet is not live).
 // S1: one specimen in mixed mode, law constants taken from m.law1 (the kernel parameters) instead of
 // the global array; see facet_warp_kernel.
+// ra, rb: the staged rows of the facet's vertices a and b; eV: e_V of its tetrahedron.
 template <class R, int MODE, bool PF, bool S1 = false>
-__device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, int j, int slot, int64_t f, bool live,
-                                          const R4<R> &g, const R4<R> &h, const R4<R> &pp,
-                                          const R (*sv)[Stride<R>::row], const R *seV, R cs[12],
+__device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, int64_t f, bool live, const R4<R> &g,
+                                          const R4<R> &h, const R4<R> &pp, const R *ra, const R *rb, R eV, R cs[12],
                                           const LawConst<R> *lbatch = nullptr)
 {
     using T4 = R4<R>;
@@ -210,14 +210,11 @@ __device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, in
 #pragma unroll
     for (int k = 0; k < 12; ++k) cs[k] = R(0);
     } else {
-    const int e = slot >> 1;
-    const int va = (0x211000 >> (4 * e)) & 0xF;
-    const int vb = (0x332321 >> (4 * e)) & 0xF;
     R A[kRow], B[kRow];
 #pragma unroll
     for (int k = 0; k < kRow; k += E) {
-        VecT<R>::get(&A[k], &sv[4 * j + va][k]);
-        VecT<R>::get(&B[k], &sv[4 * j + vb][k]);
+        VecT<R>::get(&A[k], ra + k);
+        VecT<R>::get(&B[k], rb + k);
     }
     const V3<R> d = {B[0] - A[0], B[1] - A[1], B[2] - A[2]};
     const R inv_l = rsqrt_(dot(d, d));
@@ -262,7 +259,7 @@ __device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, in
             const R wm = e3.y - h.y / aE, wl = e3.z - h.z / aE;
             T4 o4;
             o4.x = l * sqrt(wn * wn + wm * wm + wl * wl);
-            o4.y = seV[j];
+            o4.y = eV;
             o4.z = R(0);
             o4.w = R(0);
             fout[f] = o4;
@@ -277,7 +274,7 @@ __device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, in
             tM = h.y;
             tL = h.z;
             emax = h.w;
-            facet_law(c, l, e3, de3, seV[j], tN, tM, tL, emax);
+            facet_law(c, l, e3, de3, eV, tN, tM, tL, emax);
             T4 hn;
             hn.x = tN;
             hn.y = tM;
@@ -374,7 +371,8 @@ __device__ __forceinline__ void facet_block_tile(const DeviceModel &m, const voi
     // ---- phase B: one facet
     const bool live = valid && sok[j];
     R cs[12];
-    facet_one<R, MODE, PF>(m, tet0, j, slot, f, live, g, h, pp, sv, seV, cs);
+    const int e = slot >> 1, va = (0x211000 >> (4 * e)) & 0xF, vb = (0x332321 >> (4 * e)) & 0xF;
+    facet_one<R, MODE, PF>(m, tet0, f, live, g, h, pp, sv[4 * j + va], sv[4 * j + vb], seV[j], cs);
 #pragma unroll
     for (int k = 0; k < kCon; k += E) VecT<R>::put(&scon[tid][k], &cs[k]);
     __syncthreads();
@@ -411,6 +409,36 @@ __global__ void __launch_bounds__(12 * TETS) facet_kernel(DeviceModel m, const v
 // GB300 in the loaded state of 1.82M facets: 43.1 us against 45.2 us).
 constexpr int kTileTets = 8;
 constexpr int kPlane = 6 * 4 * kTileTets + 2;
+// Where facet fi (0..95) of a tile finds its rows and its places in the planes, in elements.  Edge e = slot
+// / 2 joins local vertices va < vb; it is the ka-th edge of va and the kb-th of vb (ascending), so the
+// facet is entry 2 ka + slot % 2 of va's order, 2 kb + slot % 2 of vb's.  The five numbers come from a
+// table (one 8-byte load from L1 where computing them took about 25 integer instructions per facet: 20
+// steps of 2.0M facets 1081 -> 1051 us, same results bit for bit).
+struct FacetSlot {
+    int tet, row_a, row_b, pl_a, pl_b;
+};
+struct SlotTable {
+    uint2 v[12 * kTileTets];
+    constexpr SlotTable() : v{}
+    {
+        for (int fi = 0; fi < 12 * kTileTets; ++fi) {
+            const int j = fi / 12, slot = fi - 12 * j, e = slot >> 1, sw = slot & 1;
+            const int va = (0x211000 >> (4 * e)) & 0xF, vb = (0x332321 >> (4 * e)) & 0xF;
+            const int ka = (0x221210 >> (4 * e)) & 0xF, kb = (0x211000 >> (4 * e)) & 0xF;
+            const unsigned pa = (2 * ka + sw) * kPlane + 6 * (4 * j + va), pb = (2 * kb + sw) * kPlane + 6 * (4 * j + vb);
+            v[fi].x = pa | (pb << 12) | ((unsigned)j << 24);
+            v[fi].y = (unsigned)(4 * j + va) | ((unsigned)(4 * j + vb) << 8);
+        }
+    }
+};
+__device__ const SlotTable kSlotOf{};
+template <class R>
+__device__ __forceinline__ FacetSlot facet_slot(int fi)
+{
+    const uint2 w = __ldg(&kSlotOf.v[fi]);
+    return {(int)(w.x >> 24), (int)(w.y & 0xffu) * Stride<R>::row, (int)(w.y >> 8) * Stride<R>::row,
+            (int)(w.x & 0xfffu), (int)((w.x >> 12) & 0xfffu)};
+}
 // One 8-tetrahedron tile of the facet pass, run by one warp on its own shared rows: phases A-C below.
 // PERSIST: called from the persistent step kernel (live data through ld_live).
 template <class R, int MODE, bool PF, bool S1, bool PERSIST>
@@ -422,38 +450,30 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
     using V2 = typename VecT<R>::v2;
     const T4 *__restrict__ geo = static_cast<const T4 *>(m.geo);
     const T4 *hist = static_cast<const T4 *>(m.hist);
-    // ---- prefetch the lane's three facets
+    // the tile is whole: T is a multiple of 8.  The lane's three facets, prefetched
+    const int32_t f0 = (int32_t)tet0 * 12 + lane;  // 12 T < 2^31
     T4 g[3] = {}, h[3] = {}, pp[3] = {};
+    FacetSlot fs[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const int fi = lane + 32 * i;
-        const int64_t f = tet0 * 12 + fi;
-        if (tet0 + fi / 12 < m.T) {
-            g[i] = geo[f];
-            if (MODE != FACET_ELASTIC) h[i] = ld_live<PERSIST>(hist + f);
-            if (PF) pp[i] = static_cast<const T4 *>(m.pf)[f];
-        }
+        fs[i] = facet_slot<R>(lane + 32 * i);
+        g[i] = geo[f0 + 32 * i];
+        if (MODE != FACET_ELASTIC) h[i] = ld_live<PERSIST>(hist + f0 + 32 * i);
+        if (PF) pp[i] = static_cast<const T4 *>(m.pf)[f0 + 32 * i];
     }
     // ---- phase A
     stage_vertex<R, MODE, PERSIST>(m, vsrc, tet0, lane, sv, seV, sok);
     __syncwarp();
     // ---- phase B
+    const R *rows = &sv[0][0];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const int fi = lane + 32 * i;
-        const int j = fi / 12;
-        const bool live = tet0 + j < m.T && sok[j];
-        const int slot = fi - 12 * j;
+        const int j = fs[i].tet;
         R cs[12];
-        facet_one<R, MODE, PF, S1>(m, tet0, j, slot, tet0 * 12 + fi, live, g[i], h[i], pp[i], sv, seV, cs, lbatch);
+        facet_one<R, MODE, PF, S1>(m, tet0, f0 + 32 * i, sok[j], g[i], h[i], pp[i], rows + fs[i].row_a,
+                                   rows + fs[i].row_b, seV[j], cs, lbatch);
         if (MODE != FACET_METRIC) {
-            // edge e = slot / 2 joins local vertices va < vb; it is the ka-th edge of va and the kb-th
-            // of vb (ascending), so this facet is entry 2 ka + slot % 2 of va's order, 2 kb + slot % 2 of vb's
-            const int e = slot >> 1, sw = slot & 1;
-            const int va = (0x211000 >> (4 * e)) & 0xF, vb = (0x332321 >> (4 * e)) & 0xF;
-            const int ka = (0x221210 >> (4 * e)) & 0xF, kb = (0x211000 >> (4 * e)) & 0xF;
-            R *da = spl + (2 * ka + sw) * kPlane + 6 * (4 * j + va);
-            R *db = spl + (2 * kb + sw) * kPlane + 6 * (4 * j + vb);
+            R *da = spl + fs[i].pl_a, *db = spl + fs[i].pl_b;
 #pragma unroll
             for (int c = 0; c < 6; c += 2) {
                 *reinterpret_cast<V2 *>(da + c) = V2{cs[c], cs[c + 1]};
@@ -464,12 +484,11 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
     __syncwarp();
     // ---- phase C: task t = 12 j + 3 v + q sums components 2q, 2q+1 of vertex v over the 6 planes
     if (MODE != FACET_METRIC) {
-        R *__restrict__ tvc = static_cast<R *>(m.tvc);
+        V2 *__restrict__ tvc = reinterpret_cast<V2 *>(static_cast<R *>(m.tvc)) + f0;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const int t = lane + 32 * i;
-            const int j = t / 12;
-            if (tet0 + j < m.T && sok[j]) {
+            if (sok[fs[i].tet]) {
                 R s0 = R(0), s1 = R(0);
 #pragma unroll
                 for (int sp = 0; sp < 6; ++sp) {
@@ -477,7 +496,7 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
                     s0 += x.x;
                     s1 += x.y;
                 }
-                *reinterpret_cast<V2 *>(tvc + tet0 * 24 + 2 * t) = V2{s0, s1};
+                tvc[32 * i] = V2{s0, s1};
             }
         }
     }
