@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/ldpm.h"
+#include "ldpm_device.cuh"
 #include "ldpm_internal.h"
 
 using namespace ldpm;
@@ -181,6 +182,9 @@ void law_const(const ldpm_material &mt, double dt, LawConst<R> &c)
     c.Ed_E0 = R(mt.Ed_E0);
     c.r_s = R(mt.r_s);
     c.k_t = R(mt.k_t);
+    const double mu_d = (mt.mu0 - mt.mu_inf) * mt.sigma_N0;
+    c.bs_margin = mt.mu0 >= mt.mu_inf && mt.mu_inf >= 0 ? R(4 * 1.2e-7 * mu_d) : R(-1);
+    law_bounds(c);
     c.elastic = mt.elastic;
 }
 

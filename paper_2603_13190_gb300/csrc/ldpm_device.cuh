@@ -42,6 +42,17 @@ __device__ __forceinline__ V3<double> add_cross(V3<double> w, V3<double> a, V3<d
     return {fma(a.y, b.z, fma(-a.z, b.y, w.x)), fma(a.z, b.x, fma(-a.x, b.z, w.y)), fma(a.x, b.y, fma(-a.y, b.x, w.z))};
 }
 
+// Operations with their rounding pinned: the compiler neither contracts nor splits them, so code that is
+// rearranged around them keeps its results bit for bit.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float div_fast(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double div_fast(double a, double b) { return a / b; }
+
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
 
@@ -77,6 +88,21 @@ __device__ __forceinline__ void tangent_frame(V3<R> n, V3<R> &m, V3<R> &l)
     l = {b, sgn + n.y * n.y * a, -n.y};
 }
 
+// Constants of the bounds below which the law's boundaries cannot be reached (facet_law_vjp), from sigma_t,
+// 4 alpha / r_st^2, sigma_s and r_s / alpha.  sigma_0(omega) = 2 sigma_t / D with D = s + sqrt(s^2 + k (1 -
+// s^2)), s = sin omega in [0, 1], k = 4 alpha / r_st^2, so D <= 1 + sqrt(max(1, k)).  sigma_bs(t_N) >= sigma_s
+// for t_N <= 0 where mu_0 >= mu_inf >= 0 (bs_margin >= 0 then; otherwise there is no bound), lowered by 1e-5
+// and by 4 FP32 ulp of the terms that cancel in it.
+template <class R>
+__host__ __device__ __forceinline__ void law_bounds(LawConst<R> &c)
+{
+    const R k = c.four_alpha_over_r2;
+    c.inv_s0 = (R(1) + sqrt(k > R(1) ? k : R(1))) / (R(2) * c.sigma_t);
+    c.hs = c.r_s * c.inv_alpha;
+    const R b = R(1.0 - 1e-5) * c.sigma_s - c.bs_margin;
+    c.sigma_bs_min2 = c.bs_margin >= R(0) && b > R(0) ? b * b : R(-1);
+}
+
 // Constants of the law for a facet with its own E0, alpha, sigma_t: the ones that depend on them are
 // rebuilt from the material's ratios.
 template <class R>
@@ -96,6 +122,7 @@ __device__ __forceinline__ LawConst<R> facet_params(const LawConst<R> &c, R E0, 
     p.eV0 = c.kc3 * p.ec0;
     p.Ed = c.Ed_E0 * E0;
     p.sigma_s = c.r_st * sigma_t;
+    law_bounds(p);
     return p;
 }
 
