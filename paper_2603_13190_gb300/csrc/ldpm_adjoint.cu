@@ -1114,27 +1114,22 @@ __global__ void __launch_bounds__(256) grad_to_user_kernel(const double *__restr
     if (b) atomicOr(bad, b);
 }
 
-// One thread per particle: jacc[p] += sum_d (-c_pd) R_pd(t_n) after forward step n, where on a fixed
-// DOF R = -f and on a prescribed one R = m vb (ramp(t_n + dt/2) - ramp(t_n - dt/2)) / dt - f.
-__global__ void __launch_bounds__(256) objective_kernel(DeviceModel m, AdjointModel a)
+// One thread per constrained DOF with a seed: jacc[k] += -c R(t_n) after forward step n, where on a fixed DOF
+// R = -f and on a prescribed one R = m vb (ramp(t_n + dt/2) - ramp(t_n - dt/2)) / dt - f.  (One thread per
+// particle, with its six DOFs in turn, took 7 us a step whatever the size: a chain of dependent loads.)
+__global__ void __launch_bounds__(128) objective_kernel(DeviceModel m, AdjointModel a)
 {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= m.N) return;
-    const double *pc = m.pconst + 8 * p;
-    const uint64_t bc = (uint64_t)__double_as_longlong(pc[6]);
-    if (bc == 0) return;
-    const SpecDyn &S = m.spec[(int)__double_as_longlong(pc[7])];
-    const double t = (double)(*m.step) * S.dt;
-    const double dr = (ramp(t + S.half_dt, S.inv_ramp) - ramp(t - S.half_dt, S.inv_ramp)) * S.inv_dt;
-    double acc = 0.0;
-    for (int d = 0; d < 6; ++d) {
-        const int mask = (int)((bc >> (8 * d)) & 0xffu);
-        if (mask == 0) continue;
-        double R_ = -m.pdyn[8 * p + d];
-        if (mask == 2) R_ += m.bc_vm[6 * p + d] * dr;
-        acc -= a.cseed[6 * p + d] * R_;
+    const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (k >= a.n_obj) return;
+    const ObjectiveDof o = a.obj[k];
+    const double f = m.pdyn[o.f];
+    double R_ = -f;
+    if (o.mvb != 0.0) {
+        const SpecDyn &S = m.spec[0];
+        const double t = (double)(*m.step) * S.dt;
+        R_ += o.mvb * ((ramp(t + S.half_dt, S.inv_ramp) - ramp(t - S.half_dt, S.inv_ramp)) * S.inv_dt);
     }
-    a.jacc[p] += acc;
+    a.jacc[k] -= o.c * R_;
 }
 
 // Test hook: the law and its VJP on independent rows (layouts in ldpm_internal.h).
@@ -1235,7 +1230,7 @@ cudaError_t launch_grad_to_user(const double *src, const int32_t *umap, int64_t 
 
 cudaError_t launch_objective(const DeviceModel &m, const AdjointModel &a, cudaStream_t s)
 {
-    if (m.N > 0) objective_kernel<<<(unsigned)((m.N + 255) / 256), 256, 0, s>>>(m, a);
+    if (a.n_obj > 0) objective_kernel<<<(unsigned)((a.n_obj + 127) / 128), 128, 0, s>>>(m, a);
     return cudaGetLastError();
 }
 

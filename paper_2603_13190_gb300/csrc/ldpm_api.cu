@@ -214,6 +214,7 @@ struct ldpm_ctx {
     std::vector<double> x_int;     // [N][3] internal order
     std::vector<double> inv_mass;  // [N][6]
     std::vector<double> pconst_h;  // [N][8]
+    std::vector<double> bc_vm_h;   // [N][6] the host's copy of bc_vm
     double *d_partial = nullptr, *h_out18 = nullptr;  // energy read-back: block sums; pinned result
     unsigned *d_ticket = nullptr;       // block counter of the energy reduction
     int32_t *d_umap = nullptr;          // caller's facets of all specimens, concatenated: 2 f + orientation flip
@@ -1011,6 +1012,7 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
     CU(cudaMemcpy(dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dm.bc_vel, H.bc_vel.data(), H.bc_vel.size() * sizeof(double), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dm.bc_vm, H.bc_vm.data(), H.bc_vm.size() * sizeof(double), cudaMemcpyHostToDevice));
+    h->bc_vm_h = std::move(H.bc_vm);
     CU(cudaMemcpy(dm.tet, H.tet.data(), H.tet.size() * sizeof(int4), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dm.row, H.row.data(), H.row.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     {
@@ -1358,12 +1360,17 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
     int rc;
     // c = -seed / K on constrained DOFs (internal order)
     std::vector<double> c(6 * (size_t)N, 0.0);
+    std::vector<ObjectiveDof> obj;
     for (int32_t i = 0; i < S.N; ++i) {
         const size_t P = (size_t)S.p0 + S.inv_p[i];
         uint64_t bc;
         std::memcpy(&bc, &h->pconst_h[8 * P + 6], 8);
         for (int d = 0; d < 6; ++d)
-            if ((bc >> (8 * d)) & 0xffu) c[6 * P + d] = -seed[6 * (size_t)i + d] / (double)K;
+            if (const unsigned mk = (bc >> (8 * d)) & 0xffu) {
+                const double cd = -seed[6 * (size_t)i + d] / (double)K;
+                c[6 * P + d] = cd;
+                if (cd != 0.0) obj.push_back({(int64_t)(8 * P + d), cd, mk == 2 ? h->bc_vm_h[6 * P + d] : 0.0});
+            }
     }
     const int64_t nseg = (K + C - 1) / C;
     const size_t stride = slot_stride(h);
@@ -1386,7 +1393,8 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
         return at;
     };
     const size_t o_ckpt = part(stride * (size_t)(nseg + 1)), o_snap = part(snap_stride * (size_t)std::min(C, K)),
-                 o_c = part(n6), o_Q = part(n6), o_U = part(n6), o_j = part((size_t)N * sizeof(double)), o_af = part(af),
+                 o_c = part(n6), o_Q = part(n6), o_U = part(n6), o_j = part(obj.size() * sizeof(double)),
+                 o_o = part(obj.size() * sizeof(ObjectiveDof)), o_af = part(af),
                  o_h = part(hb), o_g = part(hb), o_t = part(4 * (size_t)Fint * sizeof(R)),
                  o_s = part(mixed ? 4 * (size_t)Fint * sizeof(double) : 0), o_bad = part(sizeof(int32_t));
     char *ws = nullptr;
@@ -1413,6 +1421,8 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
     a.Qbar = (double *)(ws + o_Q);
     a.Ubar = (double *)(ws + o_U);
     a.jacc = (double *)(ws + o_j);
+    a.obj = (const ObjectiveDof *)(ws + o_o);
+    a.n_obj = (int32_t)obj.size();
     a.af = ws + o_af;
     a.adj_h = ws + o_h;
     a.gacc = ws + o_g;
@@ -1420,7 +1430,10 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
     if (mixed) a.gsum = (double *)(ws + o_s);
     int32_t *d_bad = (int32_t *)(ws + o_bad);
     CU(cudaMemcpyAsync(a.cseed, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    CU(cudaMemsetAsync(a.jacc, 0, (size_t)N * sizeof(double), h->stream));
+    if (!obj.empty()) {
+        CU(cudaMemcpyAsync(ws + o_o, obj.data(), obj.size() * sizeof(ObjectiveDof), cudaMemcpyHostToDevice, h->stream));
+        CU(cudaMemsetAsync(a.jacc, 0, obj.size() * sizeof(double), h->stream));
+    }
     auto fwd = [&](bool objective) -> int {
         int r;
         if ((r = timed(h, 1, [&]() { return launch_facet_any(h, FACET_STEP, nullptr); })) ||
@@ -1496,8 +1509,9 @@ int adjoint_run(ldpm_ctx *h, int64_t K, int64_t C, const double *seed, double *J
         if ((rc = state_copy(h, ckpt + stride * nseg, false))) return rc;
     }
     // results
-    std::vector<double> jp((size_t)N);
-    CU(cudaMemcpyAsync(jp.data(), a.jacc, jp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    std::vector<double> jp(obj.size());
+    if (!obj.empty())
+        CU(cudaMemcpyAsync(jp.data(), a.jacc, jp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     int32_t bad = 0;
     double *outs[3] = {gE0, galpha, gsigma};
     if (grads) {
@@ -1866,6 +1880,7 @@ int ldpm_set_bc(ldpm_t h, const int32_t *mask, const double *vel, double ramp_ti
     CU(cudaMemcpy(h->dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(h->dm.bc_vel, bv.data(), bv.size() * sizeof(double), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(h->dm.bc_vm, bm.data(), bm.size() * sizeof(double), cudaMemcpyHostToDevice));
+    h->bc_vm_h = std::move(bm);
     int rc = update_law(h);
     if (rc) return rc;
     if ((rc = kick(h))) return rc;

@@ -145,12 +145,19 @@ struct PersistCtl {
 //   tvc2   [T][4][12] R  per tetrahedron vertex: sums of the facets' displacement adjoints (6) and
 //          velocity adjoints (6)
 //   Qbar, Ubar [N][6] f64  adjoints of q_n and v_{n-1/2}
+// A constrained DOF with a seed: its place in pdyn, its c, and mass x prescribed velocity (0 if fixed).
+struct ObjectiveDof {
+    int64_t f;
+    double c, mvb;
+};
 struct AdjointModel {
     const void *snap_p = nullptr, *snap_h = nullptr;
     void *af = nullptr, *adj_h = nullptr, *gacc = nullptr, *tvc2 = nullptr;
     double *Qbar = nullptr, *Ubar = nullptr, *cseed = nullptr;
     double *gsum = nullptr;  // [12T][4] FP64 totals (mixed mode: gacc is folded here per segment)
-    double *jacc = nullptr;  // [N] per-particle shares of the objective, summed over the forward steps
+    const ObjectiveDof *obj = nullptr;  // [n_obj]
+    int32_t n_obj = 0;
+    double *jacc = nullptr;  // [n_obj] their shares of the objective, summed over the forward steps
     int32_t reload = 0;      // 1 if some specimen has k_t > 0 (the reload rule's derivative is needed)
 };
 
@@ -214,8 +221,8 @@ cudaError_t launch_adjoint_fold(const DeviceModel &m, const AdjointModel &a, cud
 // of *bad (0 before) is set if a value of component c is not finite.
 cudaError_t launch_grad_to_user(const double *src, const int32_t *umap, int64_t n, double *out3, int32_t *bad,
                                 cudaStream_t s);
-// After a forward step (node forces f_n in pdyn, step counter n): jacc[p] += sum_d seed_pd R_pd(t_n) / K
-// with seed / K = -c, i.e. the particle's share of the objective.
+// After a forward step (node forces f_n in pdyn, step counter n): jacc[k] += seed R(t_n) / K with seed / K =
+// -c, the share of each of the a.n_obj constrained DOFs in the objective.
 cudaError_t launch_objective(const DeviceModel &m, const AdjointModel &a, cudaStream_t s);
 // Device evaluation of the facet law and its vector-Jacobian product on independent inputs:
 // in [n][16] = l, e(3), de(3), eV, t_old(3), e_max_old, E0, alpha, sigma_t, 0; adj_out [n][4];
