@@ -399,16 +399,16 @@ __global__ void __launch_bounds__(12 * TETS) facet_kernel(DeviceModel m, const v
 // independently of the other warps.  Same arithmetic and summation order as facet_kernel<.., 8, ..>.
 // The facets' contributions are stored vertex-major: plane s (0..5) holds, for every vertex of the
 // tile, the contribution of the s-th facet in that vertex's fixed summation order (its 3 edges
-// ascending, each edge's two facets in slot order), 6 values per vertex.  The vertex sum of
-// components 2q, 2q+1 of vertex v of tetrahedron j (task t = 12 j + 3 v + q) then reads word 2t of
-// each plane: contiguous for the lanes, free of bank conflicts.  Planes are kPlane words apart (192
-// plus 2, so that the facets' stores into different planes fall on different banks).
+// ascending, each edge's two facets in slot order), 6 values per vertex.  The sums of a tile's 192
+// share values then read each plane in 16-byte vectors, contiguous for the lanes and free of bank
+// conflicts.  Planes are kPlane words apart: 192 plus 20, so that vectors stay aligned and the facets'
+// stores into different planes fall on different banks (72 wavefronts per tile, as few as any stride).
 // With one specimen (S1) the law constants are read from the kernel's own parameters (m is a
 // __grid_constant__, so taking its address makes no copy): there they are operands of the
 // instructions that use them, where the global array costs a load per use and facet (measured on
 // GB300 in the loaded state of 1.82M facets: 43.1 us against 45.2 us).
 constexpr int kTileTets = 8;
-constexpr int kPlane = 6 * 4 * kTileTets + 2;
+constexpr int kPlane = 6 * 4 * kTileTets + 20;
 // Where facet fi (0..95) of a tile finds its rows and its places in the planes, in elements.  Edge e = slot
 // / 2 joins local vertices va < vb; it is the ka-th edge of va and the kb-th of vb (ascending), so the
 // facet is entry 2 ka + slot % 2 of va's order, 2 kb + slot % 2 of vb's.  The five numbers come from a
@@ -466,11 +466,13 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
     __syncwarp();
     // ---- phase B
     const R *rows = &sv[0][0];
+    // bit j: tetrahedron j is not padding
+    const unsigned okm = __ballot_sync(0xffffffffu, lane < kTileTets && sok[lane & (kTileTets - 1)] != 0);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const int j = fs[i].tet;
         R cs[12];
-        facet_one<R, MODE, PF, S1>(m, tet0, f0 + 32 * i, sok[j], g[i], h[i], pp[i], rows + fs[i].row_a,
+        facet_one<R, MODE, PF, S1>(m, tet0, f0 + 32 * i, (okm >> j) & 1u, g[i], h[i], pp[i], rows + fs[i].row_a,
                                    rows + fs[i].row_b, seV[j], cs, lbatch);
         if (MODE != FACET_METRIC) {
             R *da = spl + fs[i].pl_a, *db = spl + fs[i].pl_b;
@@ -482,21 +484,30 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
         }
     }
     __syncwarp();
-    // ---- phase C: task t = 12 j + 3 v + q sums components 2q, 2q+1 of vertex v over the 6 planes
+    // ---- phase C: the tile's 192 share values, four per lane and round, summed over the 6 planes (10
+    // steps of 11.4M facets 2537 -> 2500 us against three rounds of two values)
     if (MODE != FACET_METRIC) {
-        V2 *__restrict__ tvc = reinterpret_cast<V2 *>(static_cast<R *>(m.tvc)) + f0;
+        using V4 = R4<R>;
+        V4 *__restrict__ tvc = reinterpret_cast<V4 *>(static_cast<R *>(m.tvc)) + (int32_t)tet0 * 6 + lane;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
+        for (int i = 0; i < 2; ++i) {
             const int t = lane + 32 * i;
-            if (sok[fs[i].tet]) {
-                R s0 = R(0), s1 = R(0);
+            if ((i == 0 || lane < 16) && ((okm >> ((t * 43) >> 8)) & 1u)) {  // t / 6
+                const V4 *src = reinterpret_cast<const V4 *>(spl) + t;
+                V4 s = src[0];
+                s.x = R(0) + s.x;
+                s.y = R(0) + s.y;
+                s.z = R(0) + s.z;
+                s.w = R(0) + s.w;
 #pragma unroll
-                for (int sp = 0; sp < 6; ++sp) {
-                    const V2 x = *reinterpret_cast<const V2 *>(spl + sp * kPlane + 2 * t);
-                    s0 += x.x;
-                    s1 += x.y;
+                for (int sp = 1; sp < 6; ++sp) {
+                    const V4 x = src[sp * (kPlane / 4)];
+                    s.x += x.x;
+                    s.y += x.y;
+                    s.z += x.z;
+                    s.w += x.w;
                 }
-                tvc[32 * i] = V2{s0, s1};
+                tvc[32 * i] = s;
             }
         }
     }
