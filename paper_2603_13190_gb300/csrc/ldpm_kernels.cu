@@ -195,7 +195,7 @@ __device__ __forceinline__ void stage_vertex(const DeviceModel &m, const void *_
 // S1: one specimen in mixed mode, law constants taken from m.law1 (the kernel parameters) instead of
 // the global array; see facet_warp_kernel.
 // ra, rb: the staged rows of the facet's vertices a and b; eV: e_V of its tetrahedron.
-template <class R, int MODE, bool PF, bool S1 = false>
+template <class R, int MODE, bool PF, bool S1 = false, bool STREAM = false>
 __device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, int64_t f, bool live, const R4<R> &g,
                                           const R4<R> &h, const R4<R> &pp, const R *ra, const R *rb, R eV, R cs[12],
                                           const LawConst<R> *lbatch = nullptr)
@@ -280,7 +280,10 @@ __device__ __forceinline__ void facet_one(const DeviceModel &m, int64_t tet0, in
             hn.y = tM;
             hn.z = tL;
             hn.w = emax;
-            hout[f] = hn;
+            if constexpr (STREAM)
+                __stcs(hout + f, hn);
+            else
+                hout[f] = hn;
         }
     }
     const R Ar = g.w;
@@ -441,7 +444,7 @@ __device__ __forceinline__ FacetSlot facet_slot(int fi)
 }
 // One 8-tetrahedron tile of the facet pass, run by one warp on its own shared rows: phases A-C below.
 // PERSIST: called from the persistent step kernel (live data through ld_live).
-template <class R, int MODE, bool PF, bool S1, bool PERSIST>
+template <class R, int MODE, bool PF, bool S1, bool PERSIST, bool STREAM = false>
 __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__restrict__ vsrc, int64_t tet0,
                                            int lane, R (*sv)[Stride<R>::row], R *spl, R *seV, int *sok,
                                            const LawConst<R> *lbatch = nullptr)
@@ -457,8 +460,13 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         fs[i] = facet_slot<R>(lane + 32 * i);
-        g[i] = geo[f0 + 32 * i];
-        if (MODE != FACET_ELASTIC) h[i] = ld_live<PERSIST>(hist + f0 + 32 * i);
+        if constexpr (STREAM) {
+            g[i] = __ldcs(geo + f0 + 32 * i);
+            h[i] = __ldcs(hist + f0 + 32 * i);
+        } else {
+            g[i] = geo[f0 + 32 * i];
+            if (MODE != FACET_ELASTIC) h[i] = ld_live<PERSIST>(hist + f0 + 32 * i);
+        }
         if (PF) pp[i] = static_cast<const T4 *>(m.pf)[f0 + 32 * i];
     }
     // ---- phase A
@@ -472,7 +480,7 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
     for (int i = 0; i < 3; ++i) {
         const int j = fs[i].tet;
         R cs[12];
-        facet_one<R, MODE, PF, S1>(m, tet0, f0 + 32 * i, (okm >> j) & 1u, g[i], h[i], pp[i], rows + fs[i].row_a,
+        facet_one<R, MODE, PF, S1, STREAM>(m, tet0, f0 + 32 * i, (okm >> j) & 1u, g[i], h[i], pp[i], rows + fs[i].row_a,
                                    rows + fs[i].row_b, seV[j], cs, lbatch);
         if (MODE != FACET_METRIC) {
             R *da = spl + fs[i].pl_a, *db = spl + fs[i].pl_b;
@@ -516,7 +524,7 @@ __device__ __forceinline__ void facet_tile(const DeviceModel &m, const void *__r
 
 // Mixed mode: capped at 80 registers (12 blocks of 2 warps per SM); without the cap the multi-specimen
 // instantiation took 93 registers and ran 8 % slower on the 97.7M-facet batch (GB300, side by side).
-template <class R, int MODE, int WPB, bool PF, bool S1>
+template <class R, int MODE, int WPB, bool PF, bool S1, bool STREAM = false>
 __global__ void __launch_bounds__(32 * WPB, sizeof(R) == 4 ? 12 : 1)
     facet_warp_kernel(const __grid_constant__ DeviceModel m, const void *__restrict__ vsrc)
 {
@@ -529,7 +537,7 @@ __global__ void __launch_bounds__(32 * WPB, sizeof(R) == 4 ? 12 : 1)
     const int64_t tet0 = ((int64_t)blockIdx.x * WPB + w) * TETS;
     if (MODE == FACET_STEP && blockIdx.x == 0 && threadIdx.x == 0) *m.step += 1;
     if (tet0 >= m.T) return;  // whole warp (T is a multiple of the tile)
-    facet_tile<R, MODE, PF, S1, false>(m, vsrc, tet0, lane, sv_[w], spl_[w], seV_[w], sok_[w]);
+    facet_tile<R, MODE, PF, S1, false, STREAM>(m, vsrc, tet0, lane, sv_[w], spl_[w], seV_[w], sok_[w]);
 }
 
 // The same for a batch of specimens, their law constants in the kernel parameters: a block of WPB
@@ -910,7 +918,7 @@ __global__ void __launch_bounds__(128) frame_kernel(DeviceModel m)
 // compensated sums run on the FP32 pipe; FP32 <-> FP64 conversions are integer operations.
 // ------------------------------------------------------------------------------------------------
 // One group of LPP lanes, particle p (all 32 lanes of the warp take part in its shuffles).
-template <class R, int MODE, int LPP, bool PERSIST>
+template <class R, int MODE, int LPP, bool PERSIST, bool STREAM = false>
 __device__ __forceinline__ void gather_group(const DeviceModel &m, int64_t p, int lane, double *__restrict__ out6)
 {
     static_assert(LPP == 8 || LPP == 16 || LPP == 32, "lanes per particle");
@@ -978,9 +986,9 @@ __device__ __forceinline__ void gather_group(const DeviceModel &m, int64_t p, in
                 for (int k = k0; k < k0 + KB && k < KT; ++k)
                     if (id[k] >= 0) {
                         const float2 *src = reinterpret_cast<const float2 *>(tvc + 6 * (int64_t)id[k]);
-                        w[k - k0][0] = ld_live<PERSIST>(src);
-                        w[k - k0][1] = ld_live<PERSIST>(src + 1);
-                        w[k - k0][2] = ld_live<PERSIST>(src + 2);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c)
+                            w[k - k0][c] = STREAM ? __ldcs(src + c) : ld_live<PERSIST>(src + c);
                     }
 #pragma unroll
                 for (int k = k0; k < k0 + KB && k < KT; ++k)
@@ -1144,12 +1152,15 @@ __device__ __forceinline__ void gather_group(const DeviceModel &m, int64_t p, in
     }
 }
 
-template <class R, int MODE, int LPP>
+// The step's pass takes the particles in descending order: the facet pass ends with the last tetrahedra, whose
+// shares are still in L2, and the next facet pass starts with the records written last (up to 1 % of a step).
+template <class R, int MODE, int LPP, bool STREAM = false>
 __global__ void __launch_bounds__(64, sizeof(R) == 4 ? 20 : 1) gather_kernel(DeviceModel m, double *__restrict__ out6)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / LPP) + lane / LPP;
-    gather_group<R, MODE, LPP, false>(m, p, lane, out6);
+    const int64_t blk = MODE == GATHER_STEP_MID ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int64_t p = ((blk * blockDim.x + threadIdx.x) >> 5) * (32 / LPP) + lane / LPP;
+    gather_group<R, MODE, LPP, false, STREAM>(m, p, lane, out6);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1615,6 +1626,14 @@ __global__ void hist_from_user_kernel(DeviceModel m, const double *__restrict__ 
     static_cast<R4<R> *>(m.hist)[f] = h;
 }
 
+// Whether the mixed step reads geometry, history and (in the particle pass) the shares, and writes the history,
+// with the streaming hint.  They pass through once per step; where the model's arrays (about 75 bytes per
+// facet) are around the size of L2 the hint leaves L2 to what both passes share (records, slot tables):
+// 2.0M facets, 20 steps 830 -> 795 us.  Where they are several times L2 nothing survives a pass anyway and
+// marking the shares first for eviction only sends them to memory: 11.4M facets, 10 steps 2383 -> 2475 us;
+// 12 specimens of 6.1M facets together, 2175 -> 2230 us.  The line is drawn at 4M facets.
+bool stream_hints(const DeviceModel &m) { return 12 * (int64_t)m.T <= 4000000; }
+
 template <class R, int MODE, bool PF>
 cudaError_t launch_facet_pf(const DeviceModel &m, const void *pst, cudaStream_t s, const BatchLaw *bl)
 {
@@ -1628,6 +1647,12 @@ cudaError_t launch_facet_pf(const DeviceModel &m, const void *pst, cudaStream_t 
             constexpr int WPB = 2;
             const int64_t tiles = (m.T + kTileTets - 1) / kTileTets;
             const unsigned nb = (unsigned)((tiles + WPB - 1) / WPB);
+            if constexpr (MODE == FACET_STEP) {
+                if (m.n_spec == 1 && stream_hints(m)) {
+                    facet_warp_kernel<R, MODE, WPB, PF, true, true><<<nb, 32 * WPB, 0, s>>>(m, pst);
+                    return cudaGetLastError();
+                }
+            }
             if (m.n_spec == 1)
                 facet_warp_kernel<R, MODE, WPB, PF, true><<<nb, 32 * WPB, 0, s>>>(m, pst);
             else if (bl && bl->n == m.n_spec)
@@ -1761,6 +1786,12 @@ cudaError_t launch_gather_lpp(const DeviceModel &m, int mode, double *out6, cuda
         gather_kernel<R, GATHER_ASSEMBLE, LPP><<<blocks, 64, 0, s>>>(m, out6);
         break;
     default:
+        if constexpr (sizeof(R) == 4 && LPP == 8) {
+            if (m.n_spec == 1 && stream_hints(m)) {
+                gather_kernel<R, GATHER_STEP_MID, LPP, true><<<blocks, 64, 0, s>>>(m, out6);
+                break;
+            }
+        }
         gather_kernel<R, GATHER_STEP_MID, LPP><<<blocks, 64, 0, s>>>(m, out6);
         break;
     }
