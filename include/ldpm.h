@@ -321,7 +321,8 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
  * every `ckpt_every` steps, and each segment but the last is recomputed once, keeping its steps'
  * inputs (the last segment's are kept during the forward run; with ckpt_every >= nsteps nothing is
  * recomputed).  Device memory: (nsteps / ckpt_every + 1) states plus ckpt_every step inputs (mixed
- * mode: 96 B per particle and 16 B per facet each).  Arithmetic in the model's precision (mixed: FP32 facet terms, FP64
+ * mode: 96 B per particle and 16 B per facet each); a workspace of up to 512 MB stays with the handle
+ * for the next call, until ldpm_destroy.  Arithmetic in the model's precision (mixed: FP32 facet terms, FP64
  * particle adjoints and gradient totals).  Derivatives at points where the law is not differentiable
  * (a switch of branch, sqrt at 0) are those of the branch the forward value takes.  With gE0, galpha
  * and gsigma_t all NULL only the forward run and J are computed.  Synchronous.
