@@ -122,8 +122,8 @@ def fp64_alu_roofline(workload: str, facet_ms: float, facets: int | None = None,
                       sm_mhz: float | None = None):
     """The FP64 facet pass against the FP64 pipe: FP64 flops of one launch (dadd + dmul + 2 dfma,
     counted by ncu on the same kernel source and workload) over the live launch time.  The count
-    depends on the loading state (which branch of the law each facet takes: 503 flops per facet on
-    the tension cube, 297.5 on the confined-compression headline), so a workload without its own
+    depends on the loading state (which branch of the law each facet takes: 190 flops per facet on
+    the tension cube, 135 on the confined-compression headline), so a workload without its own
     capture reports null rather than another workload's count scaled."""
     fl = recorded_traffic("facet_edge_kernel", workload, "fp64", "fp64_flops_per_launch")
     if fl is None or not facet_ms:
