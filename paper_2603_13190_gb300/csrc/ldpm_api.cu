@@ -272,6 +272,22 @@ int dalloc(T **p, size_t count)
     return LDPM_OK;
 }
 
+// Copy to and set of the handle's device arrays, ordered before whatever its stream runs next.  (The stream
+// does not wait for the legacy default stream, where a plain cudaMemcpy or cudaMemset runs: the copy of a
+// pageable buffer may return once it is staged, and a memset returns at once, so a kernel launched on the
+// stream after either could have read the array before it arrived.)  copy_in has read `src` when it returns.
+cudaError_t copy_in(ldpm_ctx *h, void *dst, const void *src, size_t bytes)
+{
+    if (bytes == 0) return cudaSuccess;
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(h->stream);
+}
+
+cudaError_t set_bytes(ldpm_ctx *h, void *dst, int value, size_t bytes)
+{
+    return cudaMemsetAsync(dst, value, bytes, h->stream);
+}
+
 int check_material(const ldpm_material &m)
 {
     const double v[] = {m.rho, m.E0, m.alpha, m.sigma_t, m.l_t, m.r_st, m.n_t, m.sigma_c0, m.Hc0_E0, m.Hc1_E0,
@@ -580,15 +596,15 @@ int upload_facets(ldpm_ctx *h, const HostArrays &H, int64_t Fint)
         (rc = dalloc((T4 **)&h->dm.fout, Fint)) || (rc = dalloc((R **)&h->dm.tvc, 24 * T)) ||
         (rc = dalloc((int32_t **)&h->dm.ent, std::max<int64_t>(nent, 1))))
         return rc;
-    CU(cudaMemcpy(h->dm.geo, geo.data(), Fint * sizeof(T4), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->dm.ent, ent.data(), nent * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CU(cudaMemset(h->dm.tvc, 0, 24 * T * sizeof(R)));
-    CU(cudaMemset(h->dm.hist, 0, Fint * sizeof(T4)));
-    CU(cudaMemset(h->dm.fout, 0, Fint * sizeof(T4)));
+    CU(copy_in(h, h->dm.geo, geo.data(), Fint * sizeof(T4)));
+    CU(copy_in(h, h->dm.ent, ent.data(), nent * sizeof(int32_t)));
+    CU(set_bytes(h, h->dm.tvc, 0, 24 * T * sizeof(R)));
+    CU(set_bytes(h, h->dm.hist, 0, Fint * sizeof(T4)));
+    CU(set_bytes(h, h->dm.fout, 0, Fint * sizeof(T4)));
     std::vector<LawConst<R>> law(h->sp.size());
     for (size_t s = 0; s < h->sp.size(); ++s) law_const<R>(h->sp[s].mat, h->sp[s].dt, law[s]);
     if ((rc = dalloc((LawConst<R> **)&h->dm.law, law.size()))) return rc;
-    CU(cudaMemcpy(h->dm.law, law.data(), law.size() * sizeof(LawConst<R>), cudaMemcpyHostToDevice));
+    CU(copy_in(h, h->dm.law, law.data(), law.size() * sizeof(LawConst<R>)));
     return LDPM_OK;
 }
 
@@ -597,7 +613,7 @@ int update_law(ldpm_ctx *h)
     if (h->prec == LDPM_MIXED) {
         std::vector<LawConst<float>> law(h->sp.size());
         for (size_t s = 0; s < h->sp.size(); ++s) law_const<float>(h->sp[s].mat, h->sp[s].dt, law[s]);
-        CU(cudaMemcpy(h->dm.law, law.data(), law.size() * sizeof(law[0]), cudaMemcpyHostToDevice));
+        CU(copy_in(h, h->dm.law, law.data(), law.size() * sizeof(law[0])));
         BatchLaw bl{};
         const int n = (int)h->sp.size();
         if (n > 1 && n <= kParamSpecimens) {
@@ -619,14 +635,14 @@ int update_law(ldpm_ctx *h)
     } else {
         std::vector<LawConst<double>> law(h->sp.size());
         for (size_t s = 0; s < h->sp.size(); ++s) law_const<double>(h->sp[s].mat, h->sp[s].dt, law[s]);
-        CU(cudaMemcpy(h->dm.law, law.data(), law.size() * sizeof(law[0]), cudaMemcpyHostToDevice));
+        CU(copy_in(h, h->dm.law, law.data(), law.size() * sizeof(law[0])));
     }
     std::vector<SpecDyn> sd(h->sp.size());
     for (size_t s = 0; s < h->sp.size(); ++s) {
         const double T = h->sp[s].ramp_time, dt = h->sp[s].dt;
         sd[s] = SpecDyn{dt, T, 1.0 / dt, T > 0 ? 1.0 / T : 0.0, 0.5 * dt};
     }
-    CU(cudaMemcpy(h->dm.spec, sd.data(), sd.size() * sizeof(SpecDyn), cudaMemcpyHostToDevice));
+    CU(copy_in(h, h->dm.spec, sd.data(), sd.size() * sizeof(SpecDyn)));
     return LDPM_OK;
 }
 
@@ -988,8 +1004,8 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
         (rc = dalloc(&h->d_ticket, 1)) || (rc = dalloc(&h->d_pmap, (size_t)N)) ||
         (rc = dalloc(&h->pctl.arrive, 1)) || (rc = dalloc(&h->pctl.status, 1)))
         return rc;
-    CU(cudaMemset(h->pctl.arrive, 0, sizeof(unsigned)));
-    CU(cudaMemset(h->pctl.status, 0, sizeof(int32_t)));
+    CU(set_bytes(raw, h->pctl.arrive, 0, sizeof(unsigned)));
+    CU(set_bytes(raw, h->pctl.status, 0, sizeof(int32_t)));
     {
         std::vector<int32_t> pmap((size_t)N);
         size_t base = 0;
@@ -997,24 +1013,24 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
             for (int32_t i = 0; i < S.N; ++i) pmap[base + i] = S.p0 + S.inv_p[i];
             base += S.N;
         }
-        CU(cudaMemcpy(h->d_pmap, pmap.data(), pmap.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        CU(copy_in(raw, h->d_pmap, pmap.data(), pmap.size() * sizeof(int32_t)));
     }
-    CU(cudaMemset(h->d_ticket, 0, sizeof(unsigned)));
-    CU(cudaMemcpy(h->d_umap, umap.data(), umap.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    CU(set_bytes(raw, h->d_ticket, 0, sizeof(unsigned)));
+    CU(copy_in(raw, h->d_umap, umap.data(), umap.size() * sizeof(int32_t)));
     if (H.any_fext) {
         if ((rc = dalloc(&dm.f_ext, 6 * (size_t)N))) return rc;
-        CU(cudaMemcpy(dm.f_ext, H.f_ext.data(), H.f_ext.size() * sizeof(double), cudaMemcpyHostToDevice));
+        CU(copy_in(raw, dm.f_ext, H.f_ext.data(), H.f_ext.size() * sizeof(double)));
     }
     if (h->prec == LDPM_MIXED && (rc = dalloc(&dm.pm32, (size_t)kMirror * N))) return rc;
     CU(cudaMallocHost((void **)&h->h_out18, 18 * sizeof(double)));
-    CU(cudaMemcpy(dm.pstate, H.pstate.data(), H.pstate.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dm.pdyn, H.pdyn.data(), H.pdyn.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dm.bc_vel, H.bc_vel.data(), H.bc_vel.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dm.bc_vm, H.bc_vm.data(), H.bc_vm.size() * sizeof(double), cudaMemcpyHostToDevice));
+    CU(copy_in(raw, dm.pstate, H.pstate.data(), H.pstate.size() * sizeof(double)));
+    CU(copy_in(raw, dm.pdyn, H.pdyn.data(), H.pdyn.size() * sizeof(double)));
+    CU(copy_in(raw, dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double)));
+    CU(copy_in(raw, dm.bc_vel, H.bc_vel.data(), H.bc_vel.size() * sizeof(double)));
+    CU(copy_in(raw, dm.bc_vm, H.bc_vm.data(), H.bc_vm.size() * sizeof(double)));
     h->bc_vm_h = std::move(H.bc_vm);
-    CU(cudaMemcpy(dm.tet, H.tet.data(), H.tet.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dm.row, H.row.data(), H.row.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    CU(copy_in(raw, dm.tet, H.tet.data(), H.tet.size() * sizeof(int4)));
+    CU(copy_in(raw, dm.row, H.row.data(), H.row.size() * sizeof(int32_t)));
     {
         // slot table: the first kSlotTab CSR entries of each particle, -1 after the row's end
         std::vector<int32_t> stab((size_t)kSlotTab * N, -1);
@@ -1025,11 +1041,11 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
             }
             return 0;
         });
-        CU(cudaMemcpy(dm.stab, stab.data(), stab.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        CU(copy_in(raw, dm.stab, stab.data(), stab.size() * sizeof(int32_t)));
     }
-    CU(cudaMemcpy(dm.tile_spec, H.tile_spec.data(), H.tile_spec.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CU(cudaMemset(dm.step, 0, sizeof(int64_t)));
-    CU(cudaMemset(dm.flag, 0, sizeof(int32_t)));
+    CU(copy_in(raw, dm.tile_spec, H.tile_spec.data(), H.tile_spec.size() * sizeof(int32_t)));
+    CU(set_bytes(raw, dm.step, 0, sizeof(int64_t)));
+    CU(set_bytes(raw, dm.flag, 0, sizeof(int32_t)));
     CU(launch_mirror(dm, h->stream));
     CU(cudaStreamSynchronize(h->stream));
     for (auto &S : h->sp)
@@ -1056,7 +1072,7 @@ int create_model(int n, const ldpm_geometry *geoms, const ldpm_material *mats, c
                 h->sp[s].dt = fac * 2.0 / std::sqrt(lam[s]);
             }
         if ((rc = update_law(raw))) return rc;
-        CU(cudaMemset(dm.fout, 0, Fint * h->r4size()));
+        CU(set_bytes(raw, dm.fout, 0, Fint * h->r4size()));
     }
     // the library keeps the drifted state between calls: first half kick and drift of step 0
     if ((rc = kick(raw))) return rc;
@@ -1710,12 +1726,12 @@ int ldpm_set_state(ldpm_t h, const double *q, const double *v, const double *his
             base_p += S.N;
             base_f += S.F;
         }
-        CU(cudaMemcpy(h->dm.pstate, ps.data(), ps.size() * sizeof(double), cudaMemcpyHostToDevice));
+        CU(copy_in(h, h->dm.pstate, ps.data(), ps.size() * sizeof(double)));
         CU(launch_mirror(h->dm, h->stream));
-        CU(cudaMemset(h->dm.pdyn, 0, 8 * (size_t)h->dm.N * sizeof(double)));
+        CU(set_bytes(h, h->dm.pdyn, 0, 8 * (size_t)h->dm.N * sizeof(double)));
         double *d5 = nullptr;
         if ((rc = dalloc(&d5, 5 * (size_t)Fint))) return rc;
-        cudaError_t e = cudaMemcpy(d5, h5.data(), h5.size() * sizeof(double), cudaMemcpyHostToDevice);
+        cudaError_t e = copy_in(h, d5, h5.data(), h5.size() * sizeof(double));
         if (e == cudaSuccess)
             e = h->prec == LDPM_MIXED ? launch_hist_from_user<float>(h->dm, d5, h->stream)
                                       : launch_hist_from_user<double>(h->dm, d5, h->stream);
@@ -1723,9 +1739,9 @@ int ldpm_set_state(ldpm_t h, const double *q, const double *v, const double *his
         cudaFree(d5);
         if (e != cudaSuccess || e2 != cudaSuccess)
             return fail(LDPM_E_CUDA, "history upload: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
-        CU(cudaMemcpy(h->dm.step, &step, sizeof(step), cudaMemcpyHostToDevice));
-        CU(cudaMemset(h->dm.flag, 0, sizeof(int32_t)));
-        CU(cudaMemset(h->pctl.status, 0, sizeof(int32_t)));
+        CU(copy_in(h, h->dm.step, &step, sizeof(step)));
+        CU(set_bytes(h, h->dm.flag, 0, sizeof(int32_t)));
+        CU(set_bytes(h, h->pctl.status, 0, sizeof(int32_t)));
         if ((rc = forces_from_history(h))) return rc;
         if ((rc = kick(h))) return rc;
         CU(cudaStreamSynchronize(h->stream));
@@ -1877,9 +1893,9 @@ int ldpm_set_bc(ldpm_t h, const int32_t *mask, const double *vel, double ramp_ti
     // back to the whole-step state under the old conditions, then forward under the new ones
     CU(launch_unkick(h->dm, nullptr, h->stream));
     CU(cudaStreamSynchronize(h->stream));
-    CU(cudaMemcpy(h->dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->dm.bc_vel, bv.data(), bv.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->dm.bc_vm, bm.data(), bm.size() * sizeof(double), cudaMemcpyHostToDevice));
+    CU(copy_in(h, h->dm.pconst, h->pconst_h.data(), h->pconst_h.size() * sizeof(double)));
+    CU(copy_in(h, h->dm.bc_vel, bv.data(), bv.size() * sizeof(double)));
+    CU(copy_in(h, h->dm.bc_vm, bm.data(), bm.size() * sizeof(double)));
     h->bc_vm_h = std::move(bm);
     int rc = update_law(h);
     if (rc) return rc;
@@ -1979,16 +1995,16 @@ int ldpm_load_checkpoint(ldpm_t h, const void *buf)
     const size_t n_ps = 16 * (size_t)h->dm.N * 8, n_pd = 8 * (size_t)h->dm.N * 8;
     const size_t n_h = 12 * (size_t)h->dm.T * h->r4size();
     CU(cudaStreamSynchronize(h->stream));
-    CU(cudaMemcpy(h->dm.pstate, p, n_ps, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->dm.pdyn, p + n_ps, n_pd, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->dm.hist, p + n_ps + n_pd, n_h, cudaMemcpyHostToDevice));
+    CU(copy_in(h, h->dm.pstate, p, n_ps));
+    CU(copy_in(h, h->dm.pdyn, p + n_ps, n_pd));
+    CU(copy_in(h, h->dm.hist, p + n_ps + n_pd, n_h));
     const char *q = p + n_ps + n_pd + n_h;
-    CU(cudaMemcpy(h->dm.step, q, 8, cudaMemcpyHostToDevice));
+    CU(copy_in(h, h->dm.step, q, 8));
     int64_t fl64;
     std::memcpy(&fl64, q + 8, 8);
     int32_t fl = (int32_t)fl64;
-    CU(cudaMemcpy(h->dm.flag, &fl, 4, cudaMemcpyHostToDevice));
-    CU(cudaMemset(h->pctl.status, 0, sizeof(int32_t)));
+    CU(copy_in(h, h->dm.flag, &fl, 4));
+    CU(set_bytes(h, h->pctl.status, 0, sizeof(int32_t)));
     for (size_t s = 0; s < h->sp.size(); ++s) std::memcpy(&h->sp[s].W_kin0, q + 16 + 8 * s, 8);
     CU(launch_mirror(h->dm, h->stream));
     CU(cudaStreamSynchronize(h->stream));
@@ -2130,9 +2146,9 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
         }
         if (h->prec == LDPM_MIXED) {
             std::vector<float> f32(v.begin(), v.end());
-            CU(cudaMemcpy(h->dm.pf, f32.data(), f32.size() * sizeof(float), cudaMemcpyHostToDevice));
+            CU(copy_in(h, h->dm.pf, f32.data(), f32.size() * sizeof(float)));
         } else {
-            CU(cudaMemcpy(h->dm.pf, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice));
+            CU(copy_in(h, h->dm.pf, v.data(), v.size() * sizeof(double)));
         }
         return LDPM_OK;
     } catch (const std::bad_alloc &) {
