@@ -186,6 +186,9 @@ void law_const(const ldpm_material &mt, double dt, LawConst<R> &c)
     c.bs_margin = mt.mu0 >= mt.mu_inf && mt.mu_inf >= 0 ? R(4 * 1.2e-7 * mu_d) : R(-1);
     law_bounds(c);
     c.elastic = mt.elastic;
+    // H_c = (H_c0 - H_c1) / (1 + kappa_c2 <r_DV - kappa_c1>) + H_c1 lies between H_c0 and H_c1 while the
+    // denominator is at least 1; with kappa_c2 < 0 it is not, and H_c may have any sign
+    c.hc_nonneg = mt.Hc0_E0 >= 0 && mt.Hc1_E0 >= 0 && mt.kc2 >= 0;
 }
 
 struct SpecHost {

@@ -305,7 +305,7 @@ __device__ __forceinline__ bool compression_trial64(const LawConst<double> &c, c
     const double aE = f.alpha * f.E0;
     t = {t.x + ENc * de.x, t.y + aE * de.y, t.z + aE * de.z};
     // H_c >= 0: sigma_bc >= sigma_c0, so a trial above -sigma_c0 is inside
-    if (!(c.Hc0_E0 >= 0.0 && c.Hc1_E0 >= 0.0 && order_bits(-t.x) <= order_bits(c.sigma_c0))) return true;
+    if (!(c.hc_nonneg && order_bits(-t.x) <= order_bits(c.sigma_c0))) return true;
     const float tn = fminf(d2f_trunc(t.x), 0.0f);
     // FP32 lower bound of sigma_bs: the rounding of each of its four terms is below 1e-6 of that term
     const float ss = d2f_trunc(c.r_st * f.sigma_t), md = d2f_trunc(c.mu_diff_sN0), mi = d2f_trunc(c.mu_inf) * tn,

@@ -70,6 +70,7 @@ struct LawConst {
     R k_t;  // tensile reload: traction stays zero up to e_tr = k_t (e_max - sigma_bt / E0)
     R inv_s0, hs, sigma_bs_min2, bs_margin;  // law_bounds (ldpm_device.cuh)
     int32_t elastic;
+    int32_t hc_nonneg;  // 1: H_c >= 0 in every state, so that sigma_bc >= sigma_c0
 };
 
 // Law constants of a batch of up to kParamSpecimens specimens for the kernel parameters of the FP32
