@@ -143,6 +143,19 @@ std::vector<int32_t> order_by_key(const std::vector<uint32_t> &key)
     return ia;
 }
 
+// Whether FP32 holds what the FP64 passes' filters (fracture_inside32, compression_trial64) form from the
+// parameters: products, squares and quotients of these ranges stay normal numbers.  They are far wider than any
+// unit a material is given in (MPa: 1 .. 1e5); outside them every facet's boundaries are evaluated in FP64.
+bool filter_range(const ldpm_material &m, double E0, double alpha, double sigma_t)
+{
+    auto in = [](double x, double lo, double hi) { return x >= lo && x <= hi; };
+    for (double s : {E0, sigma_t, m.r_st * sigma_t, m.sigma_c0, m.sigma_N0})
+        if (!in(s, 1e-15, 1e15)) return false;
+    return in(alpha, 1e-9, 1e9) && in(4.0 * alpha / (m.r_st * m.r_st), 1e-6, 1e6) &&
+           in(std::fabs(m.mu0 - m.mu_inf) * m.sigma_N0, 0.0, 1e15) && in(std::fabs(m.mu_inf), 0.0, 100.0) &&
+           (m.r_s == 0.0 || in(m.r_s, 1e-15, 1e9));
+}
+
 template <class R>
 void law_const(const ldpm_material &mt, double dt, LawConst<R> &c)
 {
@@ -189,6 +202,7 @@ void law_const(const ldpm_material &mt, double dt, LawConst<R> &c)
     // H_c = (H_c0 - H_c1) / (1 + kappa_c2 <r_DV - kappa_c1>) + H_c1 lies between H_c0 and H_c1 while the
     // denominator is at least 1; with kappa_c2 < 0 it is not, and H_c may have any sign
     c.hc_nonneg = mt.Hc0_E0 >= 0 && mt.Hc1_E0 >= 0 && mt.kc2 >= 0;
+    c.f32_range = filter_range(mt, E0, a, mt.sigma_t);
 }
 
 struct SpecHost {
@@ -227,6 +241,7 @@ struct ldpm_ctx {
     size_t scratch_n = 0;
     char *d_adj = nullptr;              // workspace of ldpm_adjoint, kept between calls up to kAdjointKeep bytes
     size_t adj_bytes = 0;
+    int32_t pf_range = 1;  // filter_range of the per-facet parameters (1 without them)
     std::map<int64_t, cudaGraphExec_t> graphs;
     bool prof = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -637,7 +652,10 @@ int update_law(ldpm_ctx *h)
         }
     } else {
         std::vector<LawConst<double>> law(h->sp.size());
-        for (size_t s = 0; s < h->sp.size(); ++s) law_const<double>(h->sp[s].mat, h->sp[s].dt, law[s]);
+        for (size_t s = 0; s < h->sp.size(); ++s) {
+            law_const<double>(h->sp[s].mat, h->sp[s].dt, law[s]);
+            law[s].f32_range &= h->pf_range;
+        }
         CU(copy_in(h, h->dm.law, law.data(), law.size() * sizeof(law[0])));
     }
     std::vector<SpecDyn> sd(h->sp.size());
@@ -2133,7 +2151,8 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
         if (!E0 && !alpha && !sigma_t) {
             if (h->dm.pf) cudaFree(h->dm.pf);
             h->dm.pf = nullptr;
-            return LDPM_OK;
+            h->pf_range = 1;
+            return update_law(h);
         }
         std::vector<double> v(4 * (size_t)Fint, 0.0);
         for (int64_t f = 0; f < Fint; ++f)
@@ -2142,6 +2161,11 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
             if (src[k3])
                 for (int32_t k = 0; k < S.F; ++k) v[4 * (size_t)S.fmap[k] + k3] = src[k3][k];
         for (int64_t f = 0; f < Fint; ++f) v[4 * f + 3] = 1.0 / v[4 * f + 1];
+        const int64_t outside = parallel_min(Fint, [&](int64_t f0, int64_t f1) -> int64_t {
+            for (int64_t f = f0; f < f1; ++f)
+                if (!filter_range(S.mat, v[4 * f], v[4 * f + 1], v[4 * f + 2])) return f;
+            return Fint;
+        });
         if (!h->dm.pf) {
             int rc = h->prec == LDPM_MIXED ? dalloc((float4 **)&h->dm.pf, (size_t)Fint)
                                            : dalloc((double4a **)&h->dm.pf, (size_t)Fint);
@@ -2153,7 +2177,8 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
         } else {
             CU(copy_in(h, h->dm.pf, v.data(), v.size() * sizeof(double)));
         }
-        return LDPM_OK;
+        h->pf_range = outside == Fint;
+        return update_law(h);
     } catch (const std::bad_alloc &) {
         return fail(LDPM_E_OOM, "host allocation failed");
     }

@@ -282,17 +282,25 @@ __device__ __forceinline__ float fracture_floor32(float E0, float four_a_r2, flo
     return 0.9999f * s0 * exp_(-1.0001f * H0 * over / s0);
 }
 
-// Whether the trial effective traction t surely stays below the fracture boundary.
+// Whether the trial effective traction t >= 0 surely stays below the fracture boundary.  FP32 flushes what lies
+// below 1.2e-38 and has no numbers past 3.4e38: c.f32_range keeps every stress that enters within 1e-15 .. 1e15
+// and 4 alpha / r_st^2 within 1e-6 .. 1e6, and past the elastic test the strain has to lie within 1e-12 .. 1e12
+// (its squares and 1 / e then keep cs^2 to 1e-14), so that neither can move a bound by more than its margin.
 __device__ __forceinline__ bool fracture_inside32(const LawConst<double> &c, const FacetPar64 &f, double t, double eN,
                                                   double aT2, double inv_e, double emax, double ht)
 {
+    if (!c.f32_range) return false;
     const float E0 = d2f_trunc(f.E0), st = d2f_trunc(f.sigma_t), tf = d2f_trunc(t), em = d2f_trunc(emax);
     const float al = d2f_trunc(f.alpha), k4 = al * d2f_trunc(c.four_over_r2);
     // sigma_0 >= 2 sigma_t / (1 + sqrt(max(1, 4 alpha / r_st^2))) for every omega
     const float s0min = 0.9999f * 2.0f * st / (1.0f + sqrtf(fmaxf(1.0f, k4)));
     if (E0 * em <= s0min && tf <= s0min) return true;
-    return tf <= 0.9999f * fracture_floor32(E0, k4, d2f_trunc(c.r_s) * E0 / al, st, d2f_trunc(c.n_t), d2f_trunc(eN),
-                                            d2f_trunc(aT2), d2f_trunc(inv_e), em, d2f_trunc(ht));
+    const float ie = d2f_trunc(inv_e);
+    if (!(ie >= 1e-12f && ie <= 1e12f)) return false;
+    const float low = 0.9999f * fracture_floor32(E0, k4, d2f_trunc(c.r_s) * E0 / al, st, d2f_trunc(c.n_t),
+                                                 d2f_trunc(eN), d2f_trunc(aT2), ie, em, d2f_trunc(ht));
+    // a bound of 0 (a boundary below FP32's range) holds a t of 0 only
+    return tf <= low && (low > 0.0f || order_bits(t) <= 0);
 }
 
 // Compression and friction (App. A.2, A.3) of one facet, eN <= 0.  The trial: t in, the elastic trial
@@ -305,14 +313,15 @@ __device__ __forceinline__ bool compression_trial64(const LawConst<double> &c, c
     const double aE = f.alpha * f.E0;
     t = {t.x + ENc * de.x, t.y + aE * de.y, t.z + aE * de.z};
     // H_c >= 0: sigma_bc >= sigma_c0, so a trial above -sigma_c0 is inside
-    if (!(c.hc_nonneg && order_bits(-t.x) <= order_bits(c.sigma_c0))) return true;
+    if (!(c.hc_nonneg && c.f32_range && order_bits(-t.x) <= order_bits(c.sigma_c0))) return true;
     const float tn = fminf(d2f_trunc(t.x), 0.0f);
-    // FP32 lower bound of sigma_bs: the rounding of each of its four terms is below 1e-6 of that term
+    // FP32 lower bound of sigma_bs: the rounding of each of its four terms is below 1e-6 of that term.  It is
+    // squared, so it has to lie within FP32's range for squares: c.f32_range bounds it above (1e17)
     const float ss = d2f_trunc(c.r_st * f.sigma_t), md = d2f_trunc(c.mu_diff_sN0), mi = d2f_trunc(c.mu_inf) * tn,
                 me = md * exp_(tn * d2f_trunc(c.inv_sigma_N0));
     const float low = (ss + md - mi - me) - 1e-5f * (ss + fabsf(md) + fabsf(mi) + fabsf(me));
     const float tm = d2f_trunc(t.y), tl = d2f_trunc(t.z);
-    if (!(1.00001f * (tm * tm + tl * tl) <= low * low && low > 0.0f)) return true;
+    if (!(1.00001f * (tm * tm + tl * tl) <= low * low && low >= 1e-15f)) return true;
     t.x = order_bits(t.x) > 0 ? 0.0 : t.x;
     return false;
 }

@@ -71,6 +71,7 @@ struct LawConst {
     R inv_s0, hs, sigma_bs_min2, bs_margin;  // law_bounds (ldpm_device.cuh)
     int32_t elastic;
     int32_t hc_nonneg;  // 1: H_c >= 0 in every state, so that sigma_bc >= sigma_c0
+    int32_t f32_range;  // 1: FP32 holds what the FP64 passes' filters form from the parameters
 };
 
 // Law constants of a batch of up to kParamSpecimens specimens for the kernel parameters of the FP32

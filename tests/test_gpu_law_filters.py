@@ -69,3 +69,76 @@ def test_negative_hardening_modulus():
     h = check_trajectory(mat, "compression")[2]
     assert np.sum((h[:, 0] < -0.5 * mat["sigma_c0"]) & (h[:, 0] > -0.98 * mat["sigma_c0"])) > 200
     check_gradient(mat, "compression")
+
+
+def in_unit(mat, s):
+    """The material with stresses and density in a unit 1 / s as large (the motion is the same)."""
+    return dict(mat, **{n: mat[n] * s for n in ("rho", "E0", "sigma_t", "sigma_c0", "sigma_N0")})
+
+
+@pytest.mark.parametrize("kind", ["tension", "compression"])
+@pytest.mark.parametrize("e", [-130, -70, 70, 130])
+def test_stress_units_beyond_single_precision(kind, e):
+    """At 2^+-70 the squares of the tractions, at 2^+-130 the moduli, leave the range of FP32."""
+    check_trajectory(in_unit(MAT, 2.0 ** e), kind)
+    check_gradient(in_unit(MAT, 2.0 ** e), kind)
+
+
+def test_per_facet_parameters_beyond_single_precision():
+    """Ordinary material constants, per-facet moduli and strengths below the range of FP32."""
+    mat = dict(MAT, rho=MAT["rho"] * 2.0 ** -140)
+    spec = cube()
+    bc = loading(spec, "tension")
+    par = [np.full(spec.n_facets, MAT[n] * 2.0 ** -140) for n in ("E0", "sigma_t")]
+    dt = 0.7 * oracle.Oracle(spec, MAT, 1e-7, bc).critical_dt()
+    o = oracle.Oracle(spec, mat, dt, bc)
+    o.set_facet_params(par[0], None, par[1])
+    o.step(STEPS)
+    m = ldpm.Model(spec, mat, precision="fp64", dt=dt, bc=bc)
+    m.set_facet_params(par[0], None, par[1])
+    m.step(STEPS)
+    ref = o.get_state()
+    assert (ref[2][:, 4] > 2.0 * MAT["sigma_t"] / MAT["E0"]).sum() > 10
+    for name, g, r in zip(("q", "v", "hist"), m.get_state(), ref):
+        assert_elementwise(g, r, 1e-9, name)
+    m.close()
+
+
+def test_parameters_taken_back():
+    """Out-of-range parameters set and taken back again leave the material's own law."""
+    spec, bc, dt, o = pair(MAT, "tension")
+    m = ldpm.Model(spec, MAT, precision="fp64", dt=dt, bc=bc)
+    m.set_facet_params(np.full(spec.n_facets, 1e-40), None, np.full(spec.n_facets, 1e-44))
+    m.set_facet_params(None, None, None)
+    o.step(STEPS)
+    m.step(STEPS)
+    for name, g, r in zip(("q", "v", "hist"), m.get_state(), o.get_state()):
+        assert_elementwise(g, r, 1e-9, name)
+    m.close()
+
+
+def test_vanishing_strain_of_softened_facets():
+    """Strains of 1e-27, whose squares are below the range of FP32, on facets that have softened and carry
+    traction: the boundary still depends on the direction of the strain.  Masses hold the particles still."""
+    spec = cube()
+    N, F = spec.n_particles, spec.n_facets
+    mass, inertia = np.full(N, 1e30), np.full((N, 3), 1e30)
+    rng = np.random.default_rng(8)
+    q = rng.standard_normal((N, 6)) * 1e-27
+    d = spec.x[spec.facet_pj] - spec.x[spec.facet_pi]
+    n = d / np.linalg.norm(d, axis=1)[:, None]
+    t = rng.standard_normal((F, 3))
+    t -= (t * n).sum(1)[:, None] * n
+    e0 = MAT["sigma_t"] / MAT["E0"]
+    h = np.concatenate([rng.uniform(0.2, 0.9, (F, 1)) * MAT["sigma_t"], t, e0 * rng.uniform(1.0, 8.0, (F, 1))], 1)
+    args = dict(mass=mass, inertia=inertia)
+    o = oracle.Oracle(spec, MAT, 1e-8, None, **args)
+    m = ldpm.Model(spec, MAT, precision="fp64", dt=1e-8, **args)
+    for k in (o, m):
+        k.set_state(q, np.zeros((N, 6)), h, 0)
+        k.step(1)
+    got, ref = m.get_state()[2], o.get_state()[2]
+    m.close()
+    assert np.sum(np.abs(ref[:, 0]) < 0.5 * np.abs(h[:, 0])) > 50  # capped
+    # tangential components: strains enter through differences of 1e-27 numbers exactly as larger ones would
+    assert_elementwise(got, ref, 1e-9, "hist")
