@@ -146,12 +146,13 @@ std::vector<int32_t> order_by_key(const std::vector<uint32_t> &key)
 // Whether FP32 holds what the FP64 passes' filters (fracture_inside32, compression_trial64) form from the
 // parameters: products, squares and quotients of these ranges stay normal numbers.  They are far wider than any
 // unit a material is given in (MPa: 1 .. 1e5); outside them every facet's boundaries are evaluated in FP64.
+// n_t <= 50 keeps the rounding of FP32's powers inside the filters' margin.
 bool filter_range(const ldpm_material &m, double E0, double alpha, double sigma_t)
 {
     auto in = [](double x, double lo, double hi) { return x >= lo && x <= hi; };
     for (double s : {E0, sigma_t, m.r_st * sigma_t, m.sigma_c0, m.sigma_N0})
         if (!in(s, 1e-15, 1e15)) return false;
-    return in(alpha, 1e-9, 1e9) && in(4.0 * alpha / (m.r_st * m.r_st), 1e-6, 1e6) &&
+    return in(alpha, 1e-9, 1e9) && in(m.n_t, 0.0, 50.0) && in(4.0 * alpha / (m.r_st * m.r_st), 1e-6, 1e6) &&
            in(std::fabs(m.mu0 - m.mu_inf) * m.sigma_N0, 0.0, 1e15) && in(std::fabs(m.mu_inf), 0.0, 100.0) &&
            (m.r_s == 0.0 || in(m.r_s, 1e-15, 1e9));
 }

@@ -266,9 +266,11 @@ __device__ __forceinline__ double fracture_boundary64(const LawConst<double> &c,
     return sigma0 * exp(-H0 * over / sigma0);
 }
 
-// A lower bound of it in FP32.  The margins: 1e-4 on sigma_0, on H_0 and on the exponent, 1e-6 of e_max
-// on <e_max - e_0> and of H_s + H_t on H_0 (differences of FP32 numbers).  NaN where FP32 cannot hold
-// the operands, which the caller takes as "perhaps".
+// A lower bound of it in FP32.  The margins: 1e-4 on sigma_0 and on the exponent, 1e-6 of e_max on <e_max -
+// e_0> (a difference of FP32 numbers), 1e-4 of the larger of H_s / alpha and H_t on H_0.  H_0 lies between the
+// two and may be far below the larger one, whose rounding it carries, and that of the power is up to 1e-5 +
+// 1e-6 n_t of the difference (c.f32_range: n_t <= 50).  NaN where the operands leave FP32, which the caller
+// takes as "perhaps".
 __device__ __forceinline__ float fracture_floor32(float E0, float four_a_r2, float Hs, float sigma_t, float n_t,
                                                   float eN, float aT2, float inv_e, float emax, float ht)
 {
@@ -278,7 +280,7 @@ __device__ __forceinline__ float fracture_floor32(float E0, float four_a_r2, flo
     const float over = emax - s0 / E0 + 1e-6f * emax;
     if (over <= 0.0f) return s0;
     const float Ht = E0 * ht;
-    const float H0 = 1.0001f * (Hs + (Ht - Hs) * powpos_(atan2f(eN, saT) * (float)(2.0 / kPi), n_t)) + 1e-6f * (Hs + Ht);
+    const float H0 = Hs + (Ht - Hs) * powpos_(atan2f(eN, saT) * (float)(2.0 / kPi), n_t) + 1e-4f * fmaxf(Hs, Ht);
     return 0.9999f * s0 * exp_(-1.0001f * H0 * over / s0);
 }
 

@@ -142,3 +142,47 @@ def test_vanishing_strain_of_softened_facets():
     assert np.sum(np.abs(ref[:, 0]) < 0.5 * np.abs(h[:, 0])) > 50  # capped
     # tangential components: strains enter through differences of 1e-27 numbers exactly as larger ones would
     assert_elementwise(got, ref, 1e-9, "hist")
+
+
+@pytest.mark.parametrize("n_t,r_s,l_t", [(0.2, 0.0, 120.0), (0.2, 0.5, 120.0), (20.0, 0.5, 120.0), (20.0, 50.0, 120.0),
+                                         (50.0, 50.0, None), (400.0, 0.0, 120.0), (400.0, 50.0, 120.0), (2.0, 0.0, None)])
+def test_traction_next_to_the_fracture_boundary(n_t, r_s, l_t):
+    """Softened facets with a traction within 3e-3 to 1e-5 of the boundary on either side, near pure tension
+    (where the powers (2 omega / pi)^n_t vary most) and in mixed mode, for softening exponents up to 400, shear
+    softening far steeper than the tensile one, and l_t a thousandth above the longest edge (None)."""
+    spec = cube()
+    N, F = spec.n_particles, spec.n_facets
+    d = spec.x[spec.facet_pj] - spec.x[spec.facet_pi]
+    l = np.linalg.norm(d, axis=1)
+    mat = dict(MAT, n_t=n_t, r_s=r_s, l_t=l_t if l_t else 1.001 * l.max())
+    args = dict(mass=np.full(N, 1e30), inertia=np.full((N, 3), 1e30))
+    e0 = mat["sigma_t"] / mat["E0"]
+    o = oracle.Oracle(spec, mat, 1e-8, None, **args)
+    m = ldpm.Model(spec, mat, precision="fp64", dt=1e-8, **args)
+    rng = np.random.default_rng(12)
+    zero = np.zeros((N, 6))
+    off = rng.choice([1e-5, 5e-5, 3e-4, 1e-3, 3e-3], F) * rng.choice([-1.0, 1.0], F)
+    for shear in (1e-4, 3e-3, 0.1, 1.0):
+        q = np.zeros((N, 6))
+        q[:, :3] = spec.x @ (0.2 * e0 * (np.eye(3) + shear * rng.standard_normal((3, 3))))
+        # e_max where the boundary has fallen to exp(-0.1) .. exp(-4) of sigma_0
+        e = o.strains(q)[0].reshape(F, 3)
+        om = np.arctan2(e[:, 0], np.sqrt(mat["alpha"] * (e[:, 1] ** 2 + e[:, 2] ** 2)))
+        s0 = 2 * mat["sigma_t"] / (np.sin(om) + np.sqrt(np.sin(om) ** 2 + 4 * mat["alpha"] * (np.cos(om) / mat["r_st"]) ** 2))
+        Hs, Ht = r_s * mat["E0"] / mat["alpha"], 2 * mat["E0"] / (mat["l_t"] / l - 1)
+        H0 = Hs + (Ht - Hs) * np.maximum(2 * om / np.pi, 0) ** n_t
+        h = np.zeros((F, 5))
+        h[:, 0] = 100.0 * mat["sigma_t"]
+        h[:, 4] = s0 / mat["E0"] * np.minimum(1.0 + rng.uniform(0.1, 4.0, F) * mat["E0"] / np.maximum(H0, 1e-9), 50.0)
+        o.set_state(q, zero, h, 0)
+        o.step(1)
+        t = o.get_state()[2]  # the boundary, as the cap of a traction far above it
+        cap = np.sqrt(t[:, 0] ** 2 + (t[:, 1:4] ** 2).sum(1) / mat["alpha"])
+        h[:, 0] = np.where(t[:, 0] > 0, cap * (1.0 + off), 0.0)
+        for k in (o, m):
+            k.set_state(q, zero, h, 0)
+            k.step(1)
+        got, ref = m.get_state()[2], o.get_state()[2]
+        assert np.sum(ref[:, 0] > 1e-3 * mat["sigma_t"]) > F // 3
+        assert_elementwise(got, ref, 1e-9, "shear %g" % shear)
+    m.close()
