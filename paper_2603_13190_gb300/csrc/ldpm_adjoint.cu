@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(32 * kXWarps)
                 need[i] = compression_trial64(c, fp, de, tr);
                 const bool below = order_bits(-h.x) <= order_bits(c.sigma_c0);
                 const double ENc = below ? fp.E0 : c.Ed_E0 * fp.E0;
-                const double a_tns = order_bits(h.x + ENc * de.x) > 0 ? 0.0 : at.x;
+                const double a_tns = positive(h.x + ENc * de.x) ? 0.0 : at.x;
                 const double sdd = de.y * at.y + de.z * at.z;
                 o.ae = {0.0, 0.0, 0.0};
                 o.ade = {ENc * a_tns, aE * at.y, aE * at.z};
@@ -828,8 +828,8 @@ __global__ void __launch_bounds__(32 * kXWarps)
                 const double num = de.x * (es.x + ep.x) + fp.alpha * (de.y * (es.y + ep.y) + de.z * (es.z + ep.z));
                 const double d_eff = num / (eff + eo2 * ieo);
                 const double ts = to2 * ito + fp.E0 * d_eff;
-                const double t1 = order_bits(ts) < 0 ? 0.0 : ts;
-                const bool keep = order_bits(h.w) > order_bits(eff);
+                const double t1 = negative(ts) ? 0.0 : ts;
+                const bool keep = greater_than(h.w, eff);
                 const double em = keep ? h.w : eff;
                 need[i] = order_bits(e2) < order_bits(1e-300) || (KT && c.k_t > 0.0 && order_bits(to2) <= 0) ||
                           !fracture_inside32(c, fp, t1, es.x, a2, ie, em, ht);
@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(32 * kXWarps)
                 const double r = t1 * ie;
                 const double sT = es.y * at.y + es.z * at.z;
                 const double a_r = es.x * at.x + fp.alpha * sT, ar = fp.alpha * r;
-                const double a_ts = order_bits(ts) < 0 ? 0.0 : a_r * ie;
+                const double a_ts = negative(ts) ? 0.0 : a_r * ie;
                 const double a_de = fp.E0 * a_ts;
                 const double ko = -a_de * ieo, kt = a_ts * ito;
                 double a_eff = a_de - r * ie * a_r;

@@ -245,6 +245,15 @@ __device__ __forceinline__ void facet_law(const LawConst<R> &c, R l, V3<R> e, V3
 __device__ __forceinline__ float d2f_trunc(double x);
 // Signed integer with the order of x among numbers >= 0; negative numbers (and -0) map below 0.
 __device__ __forceinline__ long long order_bits(double x) { return __double_as_longlong(x); }
+// x > 0, x < 0 (or -0) and a > b for b >= 0 on the bit patterns, false for a NaN (of either sign) in x or a, as
+// the comparisons are: a NaN that stood above every number would pass for a large one.
+constexpr unsigned long long kInfBits = 0x7ff0000000000000ull;
+__device__ __forceinline__ bool positive(double x) { return (unsigned long long)order_bits(x) - 1 < kInfBits; }
+__device__ __forceinline__ bool negative(double x) { return order_bits(x) <= (long long)(kInfBits | (1ull << 63)); }
+__device__ __forceinline__ bool greater_than(double a, double b)
+{
+    return order_bits(a) > order_bits(b) && order_bits(a) <= (long long)kInfBits;
+}
 
 // Parameters of one facet: E0, alpha, 1 / alpha, sigma_t (the facet's own or the material's).
 struct FacetPar64 {
@@ -324,7 +333,7 @@ __device__ __forceinline__ bool compression_trial64(const LawConst<double> &c, c
     const float low = (ss + md - mi - me) - 1e-5f * (ss + fabsf(md) + fabsf(mi) + fabsf(me));
     const float tm = d2f_trunc(t.y), tl = d2f_trunc(t.z);
     if (!(1.00001f * (tm * tm + tl * tl) <= low * low && low >= 1e-15f)) return true;
-    t.x = order_bits(t.x) > 0 ? 0.0 : t.x;
+    t.x = positive(t.x) ? 0.0 : t.x;
     return false;
 }
 
@@ -349,7 +358,7 @@ __device__ __forceinline__ void compression_return64(const LawConst<double> &c, 
         }
     }
     double tn = t.x < -sigma_bc ? -sigma_bc : t.x;
-    tn = order_bits(tn) > 0 ? 0.0 : tn;
+    tn = positive(tn) ? 0.0 : tn;
     const double tau2 = t.y * t.y + t.z * t.z;
     const double sigma_bs =
         c.r_st * f.sigma_t + c.mu_diff_sN0 - c.mu_inf * tn - c.mu_diff_sN0 * exp(tn * c.inv_sigma_N0);

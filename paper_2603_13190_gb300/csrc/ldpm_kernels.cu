@@ -716,12 +716,12 @@ __device__ __forceinline__ void facet_edge_tile(const DeviceModel &m, const doub
             if (order_bits(e2) < order_bits(1e-300)) {  // e < c.tiny_strain = 1e-150: t = E e
                 const double aE = fp.alpha * fp.E0, eff = sqrt(e2);
                 t[i] = {fp.E0 * es.x, aE * es.y, aE * es.z};
-                emax[i] = order_bits(emax[i]) > order_bits(eff) ? emax[i] : eff;
+                emax[i] = greater_than(emax[i], eff) ? emax[i] : eff;
                 continue;
             }
             frac[i] = true;
             const double ie = rsqrt(e2), eff = e2 * ie;
-            const double em = order_bits(emax[i]) > order_bits(eff) ? emax[i] : eff;
+            const double em = greater_than(emax[i], eff) ? emax[i] : eff;
             const V3<double> ep = es - de;
             const double e_old = sqrt(fma(ep.x, ep.x, fp.alpha * fma(ep.y, ep.y, ep.z * ep.z)));
             const double num = fma(de.x, es.x + ep.x, fp.alpha * fma(de.y, es.y + ep.y, de.z * (es.z + ep.z)));
@@ -733,7 +733,7 @@ __device__ __forceinline__ void facet_edge_tile(const DeviceModel &m, const doub
                 if (e_tr > e_old) d_eff = eff > e_tr ? eff - e_tr : 0.0;
             }
             double tr = fma(fp.E0, d_eff, t_old);
-            tr = order_bits(tr) < 0 ? 0.0 : tr;
+            tr = negative(tr) ? 0.0 : tr;
             need[i] = !fracture_inside32(c, fp, tr, es.x, a2, ie, em, ht);
             t[i].x = tr;
             emax[i] = em;
@@ -775,7 +775,7 @@ __device__ __forceinline__ void facet_edge_tile(const DeviceModel &m, const doub
             }
             if (br == 0) {
                 const double sb = fracture_boundary64(ck, fp, w[1], w[2], w[3], w[4], w[5]);
-                if (order_bits(w[0]) > order_bits(sb)) w[0] = sb;
+                if (greater_than(w[0], sb)) w[0] = sb;
             } else {
                 V3<double> tr = {w[0], w[2], w[3]};
                 compression_return64(ck, fp, w[1], w[4], tr);

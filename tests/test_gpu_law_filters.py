@@ -186,3 +186,24 @@ def test_traction_next_to_the_fracture_boundary(n_t, r_s, l_t):
         assert np.sum(ref[:, 0] > 1e-3 * mat["sigma_t"]) > F // 3
         assert_elementwise(got, ref, 1e-9, "shear %g" % shear)
     m.close()
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("kind", ["tension", "compression"])
+def test_history_without_a_maximum_strain(kind, sign):
+    """A NaN e_max (of either sign) takes the facet's strain when it is next in tension, as in the oracle: it
+    does not stand for a strain above all others, which would switch softening off for good."""
+    spec, bc, dt, o = pair(MAT, kind)
+    h = np.zeros((spec.n_facets, 5))
+    h[::3, 4] = np.copysign(np.nan, sign)
+    zero = np.zeros((spec.n_particles, 6))
+    m = ldpm.Model(spec, MAT, precision="fp64", dt=dt, bc=bc)
+    for k in (o, m):
+        k.set_state(zero, zero, h, 0)
+        k.step(STEPS)
+    got, ref = m.get_state(), o.get_state()
+    m.close()
+    assert np.sum(~np.isnan(ref[2][::3, 4])) > 10  # some have been in tension
+    assert np.array_equal(np.isnan(got[2]), np.isnan(ref[2]))
+    for name, g, r in zip(("q", "v", "hist"), got, ref):
+        assert_elementwise(np.nan_to_num(g), np.nan_to_num(r), 1e-9, name)
