@@ -126,10 +126,11 @@ typedef struct {
     const double *v0;       /* [N][6] initial velocity or NULL */
     const double *f_ext;    /* [N][6] constant external nodal forces or NULL */
     int32_t device;         /* CUDA device ordinal; < 0 = the current device */
-    int32_t autotune;       /* 1: at create, time the launch shapes (tetrahedra per facet-pass block,
-                               lanes per particle) on this model and keep the fastest; 0: defaults.
-                               Results are deterministic for a given shape; the lanes per particle
-                               set the order of a particle's force sums (rounding-level effect) */
+    int32_t autotune;       /* 1: at create, time the launch shapes (tetrahedra per facet-pass block in
+                               mixed mode; lanes per particle) on this model and keep the fastest; 0: defaults.
+                               Results are deterministic for a given shape; between shapes they differ
+                               at rounding level (the lanes per particle set the order of a particle's
+                               force sums; the mixed facet pass is compiled per block size) */
 } ldpm_options;
 
 /* Create a specimen from raw geometry (copied).  Validates the mesh rules, derives facet frames,
@@ -285,7 +286,8 @@ int ldpm_batch_energy(ldpm_t h, int32_t idx, double out[4], double reaction[12])
 int ldpm_batch_metrics(ldpm_t h, int32_t idx, double *crack_opening, double *tet_volumetric_strain);
 int ldpm_batch_info(ldpm_t h, int32_t idx, int64_t info[5], double *dt);
 
-/* Launch shape in use: shape[0] tetrahedra per facet-pass block, shape[1] lanes per particle in the
+/* Launch shape in use: shape[0] tetrahedra per facet-pass block (the FP64 step's facet pass has one shape
+ * of its own; there shape[0] is that of the other facet passes), shape[1] lanes per particle in the
  * particle pass (set by defaults, the LDPM_TETS_PER_BLOCK / LDPM_GATHER_LANES environment variables
  * at create, or the autotuner).  Library service; no counterpart in the paper. */
 int ldpm_launch_shape(ldpm_t h, int32_t shape[2]);

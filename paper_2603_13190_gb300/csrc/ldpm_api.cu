@@ -798,9 +798,11 @@ int set_launch_mode(ldpm_ctx *h, int mode);
 // Launch-shape autotuner: times each candidate (tetrahedra per facet-pass block x lanes per particle)
 // on the model itself for a few steps, restoring the complete mutable state after every trial, and
 // keeps the fastest; then times that shape's graph-replayed launch pairs against the persistent launch
-// the same way and keeps the faster mode.  Results stay deterministic for the chosen shape: the facet-pass shape does not
-// change any arithmetic, the lanes per particle change the order of a particle's sums (rounding-level
-// differences between shapes).
+// the same way and keeps the faster mode.  Results stay deterministic for the chosen shape.  Between shapes they
+// differ at rounding level: the lanes per particle change the order of a particle's sums, and in mixed mode the
+// compiler contracts the multiply-adds of the warp kernel (8 tetrahedra) and the block kernel (16, 32)
+// differently (displacements to 2e-8, history to 1e-6 of the largest after 80 steps of 66k facets).  The FP64 step has one
+// facet-pass shape.
 int autotune(ldpm_ctx *h)
 {
     DeviceModel &dm = h->dm;
@@ -826,10 +828,11 @@ int autotune(ldpm_ctx *h)
     cudaEventCreate(&a);
     cudaEventCreate(&b);
     const int tets[3] = {8, 16, 32}, lanes[2] = {8, 16};
+    const int n_tets = h->prec == LDPM_MIXED ? 3 : 1;  // the FP64 step has one facet-pass shape
     float best = 1e30f;
     int bt = dm.tets_per_block, bl = dm.gather_lanes;
     cudaError_t e = save(true);
-    for (int ti = 0; ti < 3 && e == cudaSuccess && rc == 0; ++ti)
+    for (int ti = 0; ti < n_tets && e == cudaSuccess && rc == 0; ++ti)
         for (int li = 0; li < 2 && e == cudaSuccess && rc == 0; ++li) {
             dm.tets_per_block = tets[ti];
             dm.gather_lanes = lanes[li];

@@ -1663,24 +1663,23 @@ cudaError_t launch_facet_pf(const DeviceModel &m, const void *pst, cudaStream_t 
         }
     }
     if constexpr (sizeof(R) == 8 && MODE == FACET_STEP) {
-        // the FP64 step: edge tiles, unless a launch shape of 16 or 32 tetrahedra per block was asked for
-        if (tpb == 8) {
-            const int64_t tiles = (m.T + kEdgeTets - 1) / kEdgeTets;
-            facet_edge_kernel<PF><<<(unsigned)((tiles + kEdgeWarps - 1) / kEdgeWarps), 32 * kEdgeWarps, 0, s>>>(
-                m, static_cast<const double *>(pst));
-            return cudaGetLastError();
+        // the FP64 step: edge tiles whatever the launch shape, so that it has one arithmetic (the block kernel
+        // forms its sums in another order, and takes twice the time: facet_edge_tile)
+        const int64_t tiles = ((int64_t)m.T + kEdgeTets - 1) / kEdgeTets;
+        facet_edge_kernel<PF><<<(unsigned)((tiles + kEdgeWarps - 1) / kEdgeWarps), 32 * kEdgeWarps, 0, s>>>(
+            m, static_cast<const double *>(pst));
+    } else {
+        switch (tpb) {
+        case 16:
+            facet_kernel<R, MODE, 16, PF><<<blocks, 192, 0, s>>>(m, pst);
+            break;
+        case 32:
+            facet_kernel<R, MODE, 32, PF><<<blocks, 384, 0, s>>>(m, pst);
+            break;
+        default:
+            if constexpr (sizeof(R) == 8) facet_kernel<R, MODE, 8, PF><<<blocks, 96, 0, s>>>(m, pst);
+            break;
         }
-    }
-    switch (tpb) {
-    case 16:
-        facet_kernel<R, MODE, 16, PF><<<blocks, 192, 0, s>>>(m, pst);
-        break;
-    case 32:
-        facet_kernel<R, MODE, 32, PF><<<blocks, 384, 0, s>>>(m, pst);
-        break;
-    default:
-        facet_kernel<R, MODE, 8, PF><<<blocks, 96, 0, s>>>(m, pst);
-        break;
     }
     return cudaGetLastError();
 }
