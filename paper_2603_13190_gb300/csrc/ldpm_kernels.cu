@@ -1417,12 +1417,13 @@ __global__ void __launch_bounds__(256) perturb_kernel(DeviceModel m, const doubl
     if (m.pm32) write_mirror(m.pm32 + kMirror * p, d, q, ps[9 + d]);
 }
 
-// 1 / x to FP64 rounding (x normal, > 0): FP32 seed and two Newton steps, 4 FP64 instructions where the
-// division takes about 9.
+// 1 / x, x > 0, to an ulp or two: FP32 seed and two Newton steps, 4 FP64 instructions where the division takes
+// about 9.  Where x or 1 / x is not a normal number (inverse masses below 2^-1022 or from 2^1022): the division.
 __device__ __forceinline__ double recip64(double x)
 {
     // seed from the mantissa alone (in [1, 2)), so that no x leaves FP32's range
     const long long b = __double_as_longlong(x);
+    if ((unsigned)(b >> 52) - 1u >= 2044u) return 1.0 / x;
     const double mant = __longlong_as_double((b & 0xfffffffffffffll) | 0x3ff0000000000000ll);
     const double y0 = f2d_bits(__frcp_rn(d2f_trunc(mant)));
     const double y1 = fma(y0, fma(-mant, y0, 1.0), y0);
