@@ -42,7 +42,9 @@ UNIT = "facet-updates/s"
 # force re-read and the CSR gather with its moment arms and the particle state: 178 / 334 B.  The
 # headline roofline fractions use these per-unit figures; the library's own layout moves fewer bytes
 # (frames rebuilt from the staged positions, per-tetrahedron vertex shares instead of per-facet
-# forces), given beside them as the design-byte fractions.
+# forces), given beside them as the design-byte fractions.  A fraction above 1 on these figures means
+# that the pass is faster than that layout's bytes could be moved; the design-byte fraction is the share
+# of the memory roofline.
 STORED_LAYOUT_BYTES_PER_FACET = {"mixed": {"facet_pass": 101.0, "step": 178.0},
                                  "fp64": {"facet_pass": 193.0, "step": 334.0}}
 L2_BYTES = 129e6

@@ -83,7 +83,9 @@ typedef struct {
 
 /* Material parameters, Appendix A table (names follow the paper's symbols).  ldpm_create checks
  * (LDPM_E_INVALID_ARG otherwise): every value finite; rho, E0, alpha, sigma_t, l_t, r_st, sigma_c0,
- * kc3, sigma_N0, Ed_E0 > 0; n_t, k_t, r_s >= 0; kc0 >= 1; reserved == 0. */
+ * kc3, sigma_N0, Ed_E0 > 0; n_t, k_t, r_s >= 0; kc0 >= 1; reserved == 0.  FP64 steps are fastest where
+ * moduli and strengths (per-facet ones included) lie within 1e-15 .. 1e15 in the caller's unit and
+ * n_t <= 50; the results do not depend on it. */
 typedef struct {
     double rho;      /* density */
     double E0;       /* effective normal modulus */
@@ -137,7 +139,9 @@ typedef struct {
  * arms and projected areas, the lumped mass, the particle-to-facet CSR list and the Morton-ordered
  * device layout, uploads, and estimates dt if not given.  Initial state: q = 0, v = v0 (fixed DOFs
  * 0, prescribed DOFs at their prescribed velocity), zero facet history.  On success *out owns all
- * device memory.  Errors: INVALID_ARG (options, material checks), BAD_GEOMETRY, OOM, CUDA. */
+ * device memory: about 190 bytes per facet in FP64 mode (70 of them edge frames and gradients of the
+ * reference positions) or 65 in mixed mode, and 0.6 KB per particle.  Errors: INVALID_ARG (options,
+ * material checks), BAD_GEOMETRY, OOM, CUDA. */
 int ldpm_create(const ldpm_geometry *geom, const ldpm_material *mat, const ldpm_options *opt, ldpm_t *out);
 
 /* Enqueue nsteps central-difference steps (Sec. 3) on the handle's stream and return without
@@ -326,7 +330,8 @@ int ldpm_set_facet_params(ldpm_t h, const double *E0, const double *alpha, const
  * mode: 96 B per particle and 16 B per facet each); a workspace of up to 512 MB stays with the handle
  * for the next call, until ldpm_destroy.  Arithmetic in the model's precision (mixed: FP32 facet terms, FP64
  * particle adjoints and gradient totals).  Derivatives at points where the law is not differentiable
- * (a switch of branch, sqrt at 0) are those of the branch the forward value takes.  With gE0, galpha
+ * (a switch of branch, sqrt at 0) are those of the branch the forward value takes (of the neighbouring
+ * one where the value is within rounding of the switch).  With gE0, galpha
  * and gsigma_t all NULL only the forward run and J are computed.  Synchronous.
  * Errors: INVALID_ARG, OOM (checkpoint memory), UNSTABLE (non-finite state or gradient), CUDA. */
 int ldpm_adjoint(ldpm_t h, int64_t nsteps, int32_t ckpt_every, const double *seed, double *J, double *gE0,

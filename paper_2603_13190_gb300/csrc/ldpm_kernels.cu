@@ -15,6 +15,11 @@
 //                  of the next step.
 // No tensor cores (no dense contraction), no float atomics.  The passes are bound by memory latency
 // and instruction issue (the FP64 ones by the FP64 pipe) well before HBM bandwidth.
+//
+// Times of "n steps of .. facets" in the comments of these files are pairs: the same calls before and after
+// that one change, in turn in one process.  The remaining code and the calls around the steps (models in
+// flight, state read-outs) differ from comment to comment, so the two numbers of a pair compare with each
+// other only.  Times marked ncu are single launches with cold caches.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -1629,10 +1634,16 @@ __global__ void hist_from_user_kernel(DeviceModel m, const double *__restrict__ 
 
 // Whether the mixed step reads geometry, history and (in the particle pass) the shares, and writes the history,
 // with the streaming hint.  They pass through once per step; where the model's arrays (about 75 bytes per
-// facet) are around the size of L2 the hint leaves L2 to what both passes share (records, slot tables):
-// 2.0M facets, 20 steps 830 -> 795 us.  Where they are several times L2 nothing survives a pass anyway and
-// marking the shares first for eviction only sends them to memory: 11.4M facets, 10 steps 2383 -> 2475 us;
-// 12 specimens of 6.1M facets together, 2175 -> 2230 us.  The line is drawn at 4M facets.
+// facet, 126 MB of L2) are around the size of L2 the hint leaves L2 to what both passes share (records, slot
+// tables).  Where they are several times L2, or other models' steps run in between, nothing survives a pass
+// anyway and marking the shares first for eviction only sends them to memory.  10 steps in tension, without
+// and with the hint, us (compression alike):
+//   facets               0.84M       2.0M       2.6M       3.5M       4.8M       6.0M       7.5M       9.4M
+//   one model alone   279, 278   548, 524   711, 666   910, 855 1182,1118  1451,1393  1784,1745  2204,2172
+//   three in turn     197, 190   448, 438   599, 589   802, 805 1075,1096  1346,1383  1689,1742  2112,2191
+// 11.4M facets lose in both uses (2383, 2475), and so does a batch of 6.1M (2175, 2230); smaller batches were
+// not measured and go without.  The line is where the two uses balance: at 4M facets the hint takes 5 % off a
+// model stepped alone and adds 1 % where three take turns.
 bool stream_hints(const DeviceModel &m) { return 12 * (int64_t)m.T <= 4000000; }
 
 template <class R, int MODE, bool PF>
