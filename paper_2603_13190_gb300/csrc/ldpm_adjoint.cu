@@ -77,7 +77,7 @@ __device__ __forceinline__ void facet_law_vjp(const LawConst<R> &c, R l, V3<R> e
             return;
         }
         // ---- forward values (App. A.1).  Roundings pinned in the order the compiler gives facet_law's FP32
-        // form (1.35M facets, 400 steps: gradients as before these forms within 1e-6, no facet in another
+        // form (1.35M facets, 400 steps: gradients as before these forms within 3e-6, no facet in another
         // branch).  facet_law itself is not pinned, and FP64 steps evaluate the law in another form: a facet
         // within rounding of a switch of branch may be reversed in the neighbouring one.
         const R inv_e = R(1) / eeff;

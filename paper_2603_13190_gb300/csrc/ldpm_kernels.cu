@@ -1638,12 +1638,12 @@ __global__ void hist_from_user_kernel(DeviceModel m, const double *__restrict__ 
 // tables).  Where they are several times L2, or other models' steps run in between, nothing survives a pass
 // anyway and marking the shares first for eviction only sends them to memory.  10 steps in tension, without
 // and with the hint, us (compression alike):
-//   facets               0.84M       2.0M       2.6M       3.5M       4.8M       6.0M       7.5M       9.4M
-//   one model alone   279, 278   548, 524   711, 666   910, 855 1182,1118  1451,1393  1784,1745  2204,2172
-//   three in turn     197, 190   448, 438   599, 589   802, 805 1075,1096  1346,1383  1689,1742  2112,2191
-// 11.4M facets lose in both uses (2383, 2475), and so does a batch of 6.1M (2175, 2230); smaller batches were
-// not measured and go without.  The line is where the two uses balance: at 4M facets the hint takes 5 % off a
-// model stepped alone and adds 1 % where three take turns.
+//   facets           0.84M       2.0M      2.6M      3.5M       4.8M       6.0M       7.5M       9.4M      11.3M
+//   one alone     279, 278  548, 524  711, 666  910, 855 1182, 1118 1451, 1393 1784, 1745 2204, 2172 2609, 2582
+//   three in turn 197, 190  448, 438  599, 589  802, 805 1075, 1096 1346, 1383 1689, 1742 2112, 2191 2537, 2621
+// The line is where the two uses balance: at 4M facets the hint takes 5 % off a model stepped alone and adds
+// 1 % where three take turns; past it, it gives less and costs more.  A batch of 6.1M facets loses (2175,
+// 2230); smaller batches were not measured and go without.
 bool stream_hints(const DeviceModel &m) { return 12 * (int64_t)m.T <= 4000000; }
 
 template <class R, int MODE, bool PF>
